@@ -61,7 +61,7 @@ size_t storage_bytes(int storage) {
 size_t compute_bytes(int storage) { return storage == LBF_F64 ? 8 : 4; }
 
 struct Layout {
-  size_t state[2], mom, mask, phi[2], F[2], G, gphi, partials, scal, staging, total;
+  size_t state[2], mom, mask, links, dirty, phi[2], F[2], G, gphi, partials, scal, staging, total;
   long long npartials;
   size_t staging_bytes;
 };
@@ -123,6 +123,20 @@ int aligned_by(const lbf_params* p) {
                  p->lattice == LBF_D3Q27H);
 }
 
+// the axis-separated kernel is built for a single component, except D3Q27h with walls
+bool sep_built(const lbf_params* p) {
+  return !p->two_component && !p->populations && !(p->lattice == LBF_D3Q27H && p->mask != nullptr);
+}
+constexpr int kSepMinZ = 2;  // shortest z-chunk of the axis-separated kernel
+// tiles of its largest grid, over both tile heights (walls may add the masked kernel's rows)
+long long sep_max_tiles(const lbf_params* p) {
+  const int bytes = int(storage_bytes(p->storage)), Q = p->lattice == LBF_D3Q19 ? 19 : 27;
+  const bool high = p->lattice == LBF_D3Q27H;
+  const int ty = std::min(sep_config(Q, bytes, high, false).ty, sep_config(Q, bytes, high, true).ty);
+  const int zc = std::min(kSepMinZ, p->nz);
+  return (long long)grid_x(p->nx, 32 * sep_vx(bytes)) * grid_y(p->ny, ty) * ((p->nz + zc - 1) / zc);
+}
+
 bool make_layout(const lbf_params* p, Layout* L) {
   if (check_params(p) != LBF_OK) return false;
   const long long N = (long long)p->nx * p->ny * p->nz;
@@ -140,6 +154,9 @@ bool make_layout(const lbf_params* p, Layout* L) {
   L->state[1] = take(fields * N * sb);
   L->mom = p->populations ? take(10 * N * sb) : 0;
   L->mask = p->mask ? take(N) : 0;
+  const bool links = p->mask != nullptr && sep_built(p);
+  L->links = links ? take(N * sizeof(uint32_t)) : 0;
+  L->dirty = links ? take(sep_max_tiles(p)) : 0;
   if (p->two_component) {
     L->phi[0] = take(N * cb);
     L->phi[1] = take(N * cb);
@@ -156,6 +173,7 @@ bool make_layout(const lbf_params* p, Layout* L) {
   if (const int aby = aligned_by(p)) tiles = std::max(tiles, (long long)grid_x(p->nx, 32) * grid_y(p->ny, aby));
   // walls: the step may be split into two launches over row ranges (clean rows, rows near walls)
   L->npartials = std::max<long long>(tiles * gz * (p->mask != nullptr ? 2 : 1), 1024);
+  if (sep_built(p)) L->npartials = std::max(L->npartials, (p->mask ? L->npartials : 0) + sep_max_tiles(p));
   L->partials = take(size_t(L->npartials) * 8 * sizeof(double));
   L->scal = take(64 * sizeof(double));
   L->staging_bytes = std::min<size_t>(kStagingMax, size_t(11) * 8 * size_t(N));
@@ -187,6 +205,8 @@ struct lbf_ctx {
   void* state[2];
   int cur;
   uint8_t* mask_d;
+  uint32_t* links_d;   // walls: per-site links and per-tile flags of the axis-separated kernel
+  uint8_t* dirty_d;
   void* phi[2];
   void* F[2];
   void* G;
@@ -210,6 +230,17 @@ struct lbf_ctx {
   bool aligned;         // the forward kernel is the line-aligned one (TMA loads and stores)
   CUtensorMap tmap[2];  // tensor maps of the two state buffers (TMA source)
   CUtensorMap smap[2];  // tensor maps of the two state buffers (TMA store destination)
+  // the axis-separated kernel: sep.on, over all rows, or over the clean rows of a split with the masked
+  // 30-column kernel on the others (sep_split)
+  struct {
+    bool on;
+    KernelInfo tma, async;  // rows by TMA (fn null where they do not allow it), or by cp.async
+    CUtensorMap row[2], tile[2], out[2];  // maps of the two state buffers: load boxes of one row and of a
+                                          // tile's rows, store boxes
+    dim3 grid;
+    int zchunk, y_begin, y_rows;
+  } sep;
+  bool sep_split;
   bool sums_valid;
   bool unstable_seen;
   double omega, nu_l, nu_h;
@@ -409,6 +440,8 @@ FwdParams forward_params(const lbf_ctx* c, const void* src, void* dst, bool redu
   a.src = src;
   a.dst = dst;
   a.mask = c->mask_d;
+  a.links = c->links_d;
+  a.tile_dirty = c->dirty_d;
   a.force_field = c->prm.force_field;
   for (int k = 0; k < 3; ++k) a.force[k] = c->prm.force[k];
   a.omega = c->omega;
@@ -491,6 +524,53 @@ lbf_status encode_state_map(const lbf_ctx* c, const void* base, CUtensorMap* out
   return LBF_OK;
 }
 
+// 4-D map over a state buffer for the axis-separated kernel: dims (x, field, y, z), `rows` rows of all
+// 10 fields x box_x columns per box
+lbf_status encode_row_map(const lbf_ctx* c, const void* base, CUtensorMap* out, int box_x, int rows) {
+  CUtensorMapDataType dt = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
+  switch (c->storage) {
+    case LBF_F64: dt = CU_TENSOR_MAP_DATA_TYPE_FLOAT64; break;
+    case LBF_F32: dt = CU_TENSOR_MAP_DATA_TYPE_FLOAT32; break;
+    case LBF_F16: dt = CU_TENSOR_MAP_DATA_TYPE_FLOAT16; break;
+    case LBF_BF16: dt = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16; break;
+  }
+  const cuuint64_t es = storage_bytes(c->storage);
+  const cuuint64_t dims[4] = {cuuint64_t(c->nx), 10, cuuint64_t(c->ny), cuuint64_t(c->nz)};
+  const cuuint64_t strides[3] = {es * cuuint64_t(c->N), es * c->nx, es * c->nx * cuuint64_t(c->ny)};
+  const cuuint32_t box[4] = {cuuint32_t(box_x), 10, cuuint32_t(rows), 1};
+  const cuuint32_t estr[4] = {1, 1, 1, 1};
+  CUresult r = tensor_map_encoder()(out, dt, 4, const_cast<void*>(base), dims, strides, box, estr,
+                                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) return fail(LBF_ECUDA, "cuTensorMapEncodeTiled failed with code " + std::to_string(int(r)));
+  return LBF_OK;
+}
+
+// z-chunk of the axis-separated kernel: a CTA's time grows with its planes plus the two it takes in beside
+// its own and about one of start-up, and the CTAs run in waves of `resident`. Chunks longer than 96 planes
+// let the tiles drift apart until their halo rows miss L2 (D3Q19 512^3, GLUPS at 32 / 64 / 96 / 128 / 256
+// planes: FP32 70.5 / 73.1 / 73.4 / 72.9 / 72.8, FP16 96.3 / 96.7 / 95.7 / 92.2 / 83.1). Beside the rows near
+// walls of a split step the chunks leave at least two waves (min_waves): those CTAs hold SMs as well
+// (200 x 163 x 187 BF16: 24-plane chunks 55.8, 47-plane chunks, one wave, 43.2).
+int choose_zchunk_sep(int nz, long long tiles, double resident, double min_waves) {
+  int zc = nz;
+  double best = 1e30;
+  for (int chunks = 1; chunks <= nz; ++chunks) {
+    const int z = (nz + chunks - 1) / chunks;
+    if (z < std::min(kSepMinZ, nz)) break;
+    if (z > 96) continue;
+    const long long nchunks = (nz + z - 1) / z;
+    const double waves = double(tiles * nchunks) / resident;
+    // many waves run into one another: the last one costs half of itself on average
+    const double cost = (z + 3.0) * (waves <= 12.0 ? std::max(min_waves, std::ceil(waves)) : waves + 0.5);
+    if (cost < best - 1e-9) {
+      best = cost;
+      zc = z;
+    }
+  }
+  return zc;
+}
+
 // z-chunk of a launch of `tiles` x-y tiles: the CTAs of one tile column march through nz / chunks
 // planes each, restaging two planes per chunk. Large lattices: the longest chunk (16 to 64 planes)
 // that still gives at least kMinWaves waves of resident CTAs, since fewer, longer-lived CTAs start
@@ -525,8 +605,62 @@ int choose_zchunk(int nz, long long tiles, double resident) {
 }
 
 #ifndef LBF_SPLIT_ZCHUNK
-#define LBF_SPLIT_ZCHUNK 32
+#define LBF_SPLIT_ZCHUNK 8
 #endif
+
+// the side stream of a split step
+lbf_status create_side(lbf_ctx* c) {
+  int lo = 0, hi = 0;
+  LBF_CUDA(cudaDeviceGetStreamPriorityRange(&lo, &hi));
+  LBF_CUDA(cudaStreamCreateWithPriority(&c->side, cudaStreamNonBlocking, hi));  // dispatched first
+  LBF_CUDA(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
+  LBF_CUDA(cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming));
+  return LBF_OK;
+}
+
+// the longest cyclic run of clean rows (no solid site in rows y - 1, y, y + 1 at any x and z), if it is at
+// least half of all rows and two tiles of `by` rows: shortened to whole tiles of `by` such that the rows
+// left over fill whole tiles of the masked kernel, where possible
+bool clean_band(const lbf_ctx* c, const lbf_params* p, int by, int* begin, int* len) {
+  const int nx = c->nx, ny = c->ny, nz = c->nz;
+  std::vector<char> solid_row(ny, 0);
+  for (int z = 0; z < nz; ++z)
+    for (int y = 0; y < ny; ++y) {
+      if (solid_row[y]) continue;
+      const uint8_t* row = p->mask + ((long long)z * ny + y) * nx;
+      uint64_t any = 0, word;
+      int x = 0;
+      for (; x + 8 <= nx; x += 8) {
+        std::memcpy(&word, row + x, 8);
+        any |= word;
+      }
+      for (; x < nx; ++x) any |= row[x];
+      solid_row[y] = any != 0;
+    }
+  std::vector<char> clean(ny);
+  int nclean = 0;
+  for (int y = 0; y < ny; ++y) {
+    clean[y] = !(solid_row[(y + ny - 1) % ny] || solid_row[y] || solid_row[(y + 1) % ny]);
+    nclean += clean[y];
+  }
+  if (nclean == ny || nclean < ny / 2) return false;  // no solid site at all, or walls everywhere
+  // the run starts right after a row that is not clean
+  int best_begin = 0, best_len = 0;
+  for (int y = 0; y < ny; ++y) {
+    if (!clean[y] || clean[(y + ny - 1) % ny]) continue;
+    int n = 0;
+    while (n < ny && clean[(y + n) % ny]) ++n;
+    if (n > best_len) best_len = n, best_begin = y;
+  }
+  for (int n = best_len / by * by; n >= 2 * by && n >= ny / 2; n -= by)
+    if ((ny - n) % c->fwd.by == 0) {
+      best_len = n;
+      break;
+    }
+  *begin = best_begin;
+  *len = best_len;
+  return best_len >= ny / 2 && best_len >= 2 * by;
+}
 
 // Row split for walls that occupy few rows (a channel's walls): row y is clean when rows y-1, y,
 // y+1 (periodic) hold no solid site at any x and z, so every population its outputs pull comes
@@ -548,40 +682,8 @@ lbf_status setup_split(lbf_ctx* c, const lbf_params* p, const Layout& L, int sms
   const KernelInfo al = aligned_kernel_for(c->Q, c->storage, false, false, nearest);
   if (al.fn == nullptr) return LBF_OK;
   const int nx = c->nx, ny = c->ny, nz = c->nz;
-  std::vector<char> solid_row(ny, 0);
-  for (int z = 0; z < nz; ++z)
-    for (int y = 0; y < ny; ++y) {
-      if (solid_row[y]) continue;
-      const uint8_t* row = p->mask + ((long long)z * ny + y) * nx;
-      for (int x = 0; x < nx; ++x)
-        if (row[x] != 0) {
-          solid_row[y] = 1;
-          break;
-        }
-    }
-  std::vector<char> clean(ny);
-  int nclean = 0;
-  for (int y = 0; y < ny; ++y) {
-    clean[y] = !(solid_row[(y + ny - 1) % ny] || solid_row[y] || solid_row[(y + 1) % ny]);
-    nclean += clean[y];
-  }
-  if (nclean == ny || nclean < ny / 2) return LBF_OK;  // no solid site at all, or walls everywhere
-  // the longest cyclic run of clean rows starts right after a row that is not clean
   int best_begin = 0, best_len = 0;
-  for (int y = 0; y < ny; ++y) {
-    if (!clean[y] || clean[(y + ny - 1) % ny]) continue;
-    int len = 0;
-    while (len < ny && clean[(y + len) % ny]) ++len;
-    if (len > best_len) best_len = len, best_begin = y;
-  }
-  // whole tiles on both sides where possible: the clean run shrinks to a multiple of the aligned
-  // tile height such that the rows left to the masked kernel fill whole tiles of its own height
-  for (int len = best_len / al.by * al.by; len >= 2 * al.by && len >= ny / 2; len -= al.by)
-    if ((ny - len) % c->fwd.by == 0) {
-      best_len = len;
-      break;
-    }
-  if (best_len < ny / 2 || best_len < 2 * al.by) return LBF_OK;
+  if (!clean_band(c, p, al.by, &best_begin, &best_len)) return LBF_OK;
   lbf_status st;
   if ((st = prepare(al)) != LBF_OK) return st;
   int per_sm_al = 1;
@@ -603,11 +705,7 @@ lbf_status setup_split(lbf_ctx* c, const lbf_params* p, const Layout& L, int sms
   if (blocks > L.npartials) return LBF_OK;
   for (int k = 0; k < 2; ++k)
     if ((st = encode_state_map(c, c->state[k], &c->tmap_clean[k], al.box_x, al.by + 2)) != LBF_OK) return st;
-  int lo = 0, hi = 0;
-  LBF_CUDA(cudaDeviceGetStreamPriorityRange(&lo, &hi));
-  LBF_CUDA(cudaStreamCreateWithPriority(&c->side, cudaStreamNonBlocking, hi));  // dispatched first
-  LBF_CUDA(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
-  LBF_CUDA(cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming));
+  if ((st = create_side(c)) != LBF_OK) return st;
   c->fwd_clean = al;
   c->clean_begin = best_begin;
   c->clean_rows = best_len;
@@ -618,6 +716,64 @@ lbf_status setup_split(lbf_ctx* c, const lbf_params* p, const Layout& L, int sms
   c->grid_clean = gc;
   c->grid_dirty = gd;
   c->split = true;
+  return LBF_OK;
+}
+
+// Chooses the axis-separated kernel for the step, its tile and its z-chunk.
+lbf_status setup_sep(lbf_ctx* c, const lbf_params* p, const Layout& L, int sms, bool nearest, const std::string& kname) {
+  const bool forced = kname == "sep" || kname == "sepsmall";
+  if (!sep_built(p) || !(kname.empty() || forced)) return LBF_OK;
+  if (storage_bytes(c->storage) == 2 && c->nx % 2 != 0) return LBF_OK;  // no 4-byte aligned pairs of sites
+  const bool field = p->force_field != nullptr;
+  // below about 2^20 sites the tall tiles leave SMs idle: short ones (ensemble members, 524288 sites with
+  // walls and a force field: 17 us a step against 20.6)
+  const bool small = kname == "sepsmall" || (kname != "sep" && c->N < (1LL << 20));
+  const bool rows_tma = tma_eligible(c->storage, c->nx) && c->nx >= 32 * sep_vx(int(storage_bytes(c->storage)));
+  // large lattices whose rows TMA cannot take: the 30-column kernel (333 x 250 x 189: 37.9 against 33.0)
+  if (!rows_tma && !small && !forced) return LBF_OK;
+  bool walls = c->has_mask;
+  c->sep.y_begin = 0;
+  c->sep.y_rows = c->ny;
+  if (walls && kname.empty() && !small) {
+    const KernelInfo k = sep_kernel_for(c->Q, c->storage, false, field, false, nearest, small);
+    int begin = 0, len = 0;
+    if (!clean_band(c, p, k.by, &begin, &len)) return LBF_OK;  // scattered walls: the 30-column kernel
+    walls = false;
+    c->sep_split = true;
+    c->sep.y_begin = begin;
+    c->sep.y_rows = len;
+    c->dirty_begin = (begin + len) % c->ny;
+    c->dirty_rows = c->ny - len;
+    c->zchunk_dirty = std::min(LBF_SPLIT_ZCHUNK, c->nz);
+    c->grid_dirty = dim3(grid_x(c->nx, c->fwd.xout), grid_y(c->dirty_rows, c->fwd.by), (c->nz + c->zchunk_dirty - 1) / c->zchunk_dirty);
+  }
+  c->sep.async = sep_kernel_for(c->Q, c->storage, walls, field, false, nearest, small);
+  c->sep.tma = KernelInfo{nullptr, 0, 0, 0, 0};
+  if (rows_tma)
+    c->sep.tma = sep_kernel_for(c->Q, c->storage, walls, field, true, nearest, small);
+  lbf_status st;
+  if ((st = prepare(c->sep.async)) != LBF_OK || (st = prepare(c->sep.tma)) != LBF_OK) return st;
+  const KernelInfo& k = c->sep.tma.fn ? c->sep.tma : c->sep.async;
+  int resident = 1;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, k.fn, k.threads, k.smem) != cudaSuccess)
+    return fail(LBF_ECUDA, std::string("device query failed: ") + cudaGetErrorString(cudaGetLastError()));
+  const long long tiles = (long long)grid_x(c->nx, k.xout) * grid_y(c->sep.y_rows, k.by);
+  c->sep.zchunk = choose_zchunk_sep(c->nz, tiles, double(sms) * std::max(resident, 1), c->sep_split ? 2.0 : 1.0);
+  if (const char* e = std::getenv("LBF_ZCHUNK")) {
+    const int v = std::atoi(e);
+    if (v >= 1) c->sep.zchunk = std::min(c->nz, std::max(std::min(kSepMinZ, c->nz), v));
+  }
+  c->sep.grid = dim3(grid_x(c->nx, k.xout), grid_y(c->sep.y_rows, k.by), (c->nz + c->sep.zchunk - 1) / c->sep.zchunk);
+  const long long blocks = (long long)c->sep.grid.x * c->sep.grid.y * c->sep.grid.z +
+                           (c->sep_split ? (long long)c->grid_dirty.x * c->grid_dirty.y * c->grid_dirty.z : 0);
+  if (blocks > L.npartials) return fail(LBF_EINTERNAL, "partials buffer too small");
+  for (int i = 0; i < 2 && c->sep.tma.fn != nullptr; ++i)
+    if ((st = encode_row_map(c, c->state[i], &c->sep.row[i], k.box_x, 1)) != LBF_OK ||
+        (st = encode_row_map(c, c->state[i], &c->sep.tile[i], k.box_x, k.by + 2)) != LBF_OK ||
+        (st = encode_row_map(c, c->state[i], &c->sep.out[i], k.box_x, k.out_rows)) != LBF_OK)
+      return st;
+  if (c->sep_split && (st = create_side(c)) != LBF_OK) return st;
+  c->sep.on = true;
   return LBF_OK;
 }
 
@@ -653,6 +809,69 @@ lbf_status launch_split(lbf_ctx* c, const FwdParams& a, int ks) {
   return LBF_OK;
 }
 
+// the axis-separated step; *done = false (and nothing launched) where the buffers do not allow it
+lbf_status launch_sep(lbf_ctx* c, const FwdParams& a, const void* src, void* dst, bool* done) {
+  const uintptr_t us = reinterpret_cast<uintptr_t>(src), ud = reinterpret_cast<uintptr_t>(dst);
+  FwdParams as = a;
+  as.zchunk = c->sep.zchunk;
+  as.y_begin = c->sep.y_begin;
+  as.y_rows = c->sep.y_rows;
+  CUtensorMap tr, tt, to, tmd;
+  std::memset(&tr, 0, sizeof(tr));
+  std::memset(&tt, 0, sizeof(tt));
+  std::memset(&to, 0, sizeof(to));
+  std::memset(&tmd, 0, sizeof(tmd));
+  const KernelInfo* k = &c->sep.async;
+  const int ks = src == c->state[0] ? 0 : (src == c->state[1] ? 1 : -1);
+  const int kd = dst == c->state[0] ? 0 : (dst == c->state[1] ? 1 : -1);
+  lbf_status st = LBF_OK;
+  if (c->sep.tma.fn != nullptr && us % 16 == 0 && ud % 16 == 0) {  // TMA boxes start on 16-byte boundaries
+    k = &c->sep.tma;
+    if (ks >= 0) tr = c->sep.row[ks], tt = c->sep.tile[ks];
+    else if ((st = encode_row_map(c, src, &tr, k->box_x, 1)) == LBF_OK) st = encode_row_map(c, src, &tt, k->box_x, k->by + 2);
+    if (st == LBF_OK && kd >= 0) to = c->sep.out[kd];
+    else if (st == LBF_OK) st = encode_row_map(c, dst, &to, k->box_x, k->out_rows);
+    if (st != LBF_OK) return st;
+  } else if (us % (storage_bytes(c->storage) == 8 ? 8 : 4) != 0) {  // cp.async copies 4 or 8 bytes
+    return LBF_OK;
+  }
+  void* args[] = {&as, &tr, &tt, &to};
+  const dim3 block(32, k->threads / 32, 1);
+  if (!c->sep_split) {
+    LBF_CUDA(cudaLaunchKernel(k->fn, c->sep.grid, block, args, k->smem, c->stream));
+    *done = true;
+    return LBF_OK;
+  }
+  // walls in a band of rows: the rows near them on the side stream, joined at the end of the step; the
+  // two launches share the block counter, and the last block of either adds all partials
+  const KernelInfo* kw = &c->fwd;
+  if (c->tma && us % 16 == 0) {
+    if (ks >= 0) tmd = c->tmap[ks];
+    else if ((st = encode_state_map(c, src, &tmd, kw->box_x, kw->by + 2)) != LBF_OK) return st;
+  } else {
+    kw = &c->fwd_direct;
+  }
+  FwdParams aw = a;
+  const long long nw = (long long)c->grid_dirty.x * c->grid_dirty.y * c->grid_dirty.z;
+  const long long nall = nw + (long long)c->sep.grid.x * c->sep.grid.y * c->sep.grid.z;
+  aw.y_begin = c->dirty_begin;
+  aw.y_rows = c->dirty_rows;
+  aw.zchunk = c->zchunk_dirty;
+  aw.block_base = 0;
+  as.block_base = nw;
+  aw.final_blocks = as.final_blocks = nall;
+  as.mask = nullptr;  // every site of the clean rows and of their neighbour rows is fluid
+  void* argw[] = {&aw, &tmd, &tmd};
+  LBF_CUDA(cudaEventRecord(c->ev_fork, c->stream));
+  LBF_CUDA(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
+  LBF_CUDA(cudaLaunchKernel(kw->fn, c->grid_dirty, dim3(32, kw->threads / 32, 1), argw, kw->smem, c->side));
+  LBF_CUDA(cudaEventRecord(c->ev_join, c->side));
+  LBF_CUDA(cudaLaunchKernel(k->fn, c->sep.grid, block, args, k->smem, c->stream));
+  LBF_CUDA(cudaStreamWaitEvent(c->stream, c->ev_join, 0));
+  *done = true;
+  return LBF_OK;
+}
+
 lbf_status launch_forward(lbf_ctx* c, const void* src, void* dst, bool reduce) {
   if (c->pops) {
     PopParams pp = pop_params(c, src, dst, reduce);
@@ -662,6 +881,11 @@ lbf_status launch_forward(lbf_ctx* c, const void* src, void* dst, bool reduce) {
   }
   FwdParams a = forward_params(c, src, dst, reduce);
   ++c->steps_done;
+  if (c->sep.on) {
+    bool done = false;
+    const lbf_status st = launch_sep(c, a, src, dst, &done);
+    if (st != LBF_OK || done) return st;
+  }
   if (c->split) {
     const int ks = src == c->state[0] ? 0 : (src == c->state[1] ? 1 : -1);
     const int kd = dst == c->state[0] ? 0 : (dst == c->state[1] ? 1 : -1);
@@ -791,7 +1015,7 @@ int lbf_version(void) { return 1; }
 
 int lbf_kernels_per_step(const lbf_ctx* c) {
   if (c == nullptr) return 0;
-  return (c->split ? 2 : 1) + (c->two ? 2 : 0);
+  return (c->split || c->sep_split ? 2 : 1) + (c->two ? 2 : 0);
 }
 
 const char* lbf_last_error(void) { return g_last_error.c_str(); }
@@ -848,6 +1072,8 @@ lbf_status lbf_create(lbf_ctx** out, const lbf_params* params, void* workspace, 
   c->mom = c->pops ? c->ws + L.mom : nullptr;
   c->pop_grid = dim3((c->nx + kPopThreads - 1) / kPopThreads, c->ny, c->nz);
   c->mask_d = c->has_mask ? reinterpret_cast<uint8_t*>(c->ws + L.mask) : nullptr;
+  c->links_d = L.links ? reinterpret_cast<uint32_t*>(c->ws + L.links) : nullptr;
+  c->dirty_d = L.links ? reinterpret_cast<uint8_t*>(c->ws + L.dirty) : nullptr;
   for (int k = 0; k < 2; ++k) {
     c->phi[k] = c->two ? c->ws + L.phi[k] : nullptr;
     c->F[k] = c->two ? c->ws + L.F[k] : nullptr;
@@ -948,7 +1174,10 @@ lbf_status lbf_create(lbf_ctx** out, const lbf_params* params, void* workspace, 
   for (const KernelInfo* k : {&c->fwd, &c->fwd_tma30, &c->fwd_direct})
     if ((long long)grid_x(c->nx, k->xout) * grid_y(c->ny, k->by) * gz > L.npartials)
       return cleanup(fail(LBF_EINTERNAL, "partials buffer too small"));
-  if ((st = setup_split(c, params, L, sms, nearest, kname)) != LBF_OK) return cleanup(st);
+  c->sep.on = false;
+  c->sep_split = false;
+  if ((st = setup_sep(c, params, L, sms, nearest, kname)) != LBF_OK) return cleanup(st);
+  if (!c->sep.on && (st = setup_split(c, params, L, sms, nearest, kname)) != LBF_OK) return cleanup(st);
 
   cudaStream_t s = c->stream;
   if (cudaMemsetAsync(c->state[0], 0, 10 * c->N * storage_bytes(c->storage), s) != cudaSuccess ||
@@ -958,6 +1187,16 @@ lbf_status lbf_create(lbf_ctx** out, const lbf_params* params, void* workspace, 
   if (c->has_mask) {
     if (cudaMemcpyAsync(c->mask_d, params->mask, c->N, cudaMemcpyHostToDevice, s) != cudaSuccess)
       return cleanup(fail(LBF_ECUDA, "mask copy failed"));
+    if (c->sep.on && !c->sep_split) {
+      const unsigned g = blocks_for(c->N, 256);
+      if (c->Q == LBF_D3Q19)
+        k_wall_links<D3Q19><<<g, 256, 0, s>>>(c->mask_d, c->nx, c->ny, c->nz, c->links_d);
+      else
+        k_wall_links<D3Q27><<<g, 256, 0, s>>>(c->mask_d, c->nx, c->ny, c->nz, c->links_d);
+      k_tile_dirty<<<c->sep.grid, 256, 0, s>>>(c->mask_d, c->nx, c->ny, c->nz, c->sep.async.xout, c->sep.async.by,
+                                               c->sep.zchunk, c->sep.tma.fn != nullptr, c->dirty_d);
+      if (cudaGetLastError() != cudaSuccess) return cleanup(fail(LBF_ECUDA, "wall links failed"));
+    }
   }
   if (c->two) {
     const size_t cb = compute_bytes(c->storage);

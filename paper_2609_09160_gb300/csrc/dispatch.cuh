@@ -7,6 +7,7 @@
 #include "population.cuh"
 #include "stream_collide.cuh"
 #include "stream_collide_aligned.cuh"
+#include "stream_collide_sep.cuh"
 
 namespace lbf {
 
@@ -22,7 +23,8 @@ struct KernelInfo {
   int threads;      // threads per CTA
   int by;           // output rows per CTA
   int box_x;        // TMA box width in elements (0: the kernel loads without TMA)
-  int xout = 30;    // output columns per CTA: 30 (k_stream_collide) or 32 (k_stream_collide_al)
+  int xout = 30;    // output columns per CTA: 30 (k_stream_collide), 32 (k_stream_collide_al), 64 or 32 (k_stream_collide_sep)
+  int out_rows = 1; // rows per TMA store (k_stream_collide_sep)
   bool store_map = false;  // the kernel also takes a tensor map of dst (TMA stores)
 };
 
@@ -124,6 +126,51 @@ KernelInfo aligned_kernel_ls(bool mask, bool field, bool nearest) {
   }
 }
 
+// the axis-separated kernel (single component). fn == nullptr for D3Q27h with walls, which is not
+// built (its wall populations need the full basis). small: the tile for lattices that leave most of the
+// chip idle; tma: rows by TMA, else by cp.async (16-bit storage: nx must be even)
+template <class L, class S, bool SMALL, bool TMA, bool MASK, bool FF, bool RN>
+KernelInfo sep_info() {
+  constexpr SepConfig C = sep_config(L::Q, int(sizeof(S)), L::HIGH, SMALL);
+  constexpr int VX = sep_vx(int(sizeof(S)));
+  using G = SepTile<L, S, VX, C.ty, C.rp>;
+  KernelInfo k;
+  k.fn = reinterpret_cast<const void*>(&k_stream_collide_sep<L, S, SMALL, TMA, MASK, FF, RN>);
+  k.smem = sep_smem_bytes<L, S, VX, C.ty, C.rp, C.stages, MASK>();
+  k.threads = G::THREADS;
+  k.by = C.ty;
+  k.box_x = TMA ? G::XO : 0;
+  k.xout = G::XO;
+  k.out_rows = C.rp;
+  return k;
+}
+
+template <class L, class S, bool SMALL, bool RN>
+KernelInfo sep_kernel_s(bool mask, bool field, bool tma) {
+  if (mask) {
+    if constexpr (L::HIGH) {
+      return KernelInfo{nullptr, 0, 0, 0, 0};
+    } else {
+      if (field) return tma ? sep_info<L, S, SMALL, true, true, true, RN>() : sep_info<L, S, SMALL, false, true, true, RN>();
+      return tma ? sep_info<L, S, SMALL, true, true, false, RN>() : sep_info<L, S, SMALL, false, true, false, RN>();
+    }
+  }
+  if (field) return tma ? sep_info<L, S, SMALL, true, false, true, RN>() : sep_info<L, S, SMALL, false, false, true, RN>();
+  return tma ? sep_info<L, S, SMALL, true, false, false, RN>() : sep_info<L, S, SMALL, false, false, false, RN>();
+}
+
+template <class L, class S>
+KernelInfo sep_kernel_ls(bool mask, bool field, bool tma, bool nearest, bool small) {
+  if constexpr (Codec<S>::scaled) {
+    if (nearest) return small ? sep_kernel_s<L, S, true, true>(mask, field, tma) : sep_kernel_s<L, S, false, true>(mask, field, tma);
+  }
+  if constexpr (std::is_same<S, double>::value) {
+    return sep_kernel_s<L, S, false, false>(mask, field, tma);
+  } else {
+    return small ? sep_kernel_s<L, S, true, false>(mask, field, tma) : sep_kernel_s<L, S, false, false>(mask, field, tma);
+  }
+}
+
 // population-form reference kernels of lattice L, storage S (FP32/FP64 only; nulls otherwise)
 struct PopKernels {
   const void* step;     // k_pop_step
@@ -154,6 +201,7 @@ PopKernels pop_kernels_ls(bool mask, bool field) {
 #define LBF_DECLARE_TU(q, s)                                                             \
   KernelInfo forward_kernel_q##q##_s##s(bool mask, int two, bool field, bool tma, bool nearest); \
   KernelInfo aligned_kernel_q##q##_s##s(bool mask, bool field, bool nearest);                    \
+  KernelInfo sep_kernel_q##q##_s##s(bool mask, bool field, bool tma, bool nearest, bool small);  \
   PopKernels pop_kernels_q##q##_s##s(bool mask, bool field);                                        \
   KernelInfo adjoint_kernel_q##q##_s##s(bool mask);
 LBF_DECLARE_TU(19, 0)
@@ -213,6 +261,25 @@ inline KernelInfo aligned_kernel_for(int lattice, int storage, bool mask, bool f
     LBF_AL_CASE(127)
   }
 #undef LBF_AL_CASE
+  return KernelInfo{nullptr, 0, 0, 0, 0};
+}
+
+inline KernelInfo sep_kernel_for(int lattice, int storage, bool mask, bool field, bool tma, bool nearest, bool small) {
+#define LBF_SEP_CASE(q)                                                       \
+  switch (storage) {                                                         \
+    case ST_F64: return sep_kernel_q##q##_s0(mask, field, tma, nearest, small);     \
+    case ST_F32: return sep_kernel_q##q##_s1(mask, field, tma, nearest, small);     \
+    case ST_F16: return sep_kernel_q##q##_s2(mask, field, tma, nearest, small);     \
+    case ST_BF16: return sep_kernel_q##q##_s3(mask, field, tma, nearest, small);    \
+  }
+  if (lattice == 19) {
+    LBF_SEP_CASE(19)
+  } else if (lattice == 27) {
+    LBF_SEP_CASE(27)
+  } else if (lattice == 127) {
+    LBF_SEP_CASE(127)
+  }
+#undef LBF_SEP_CASE
   return KernelInfo{nullptr, 0, 0, 0, 0};
 }
 

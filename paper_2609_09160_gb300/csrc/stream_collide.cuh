@@ -44,6 +44,8 @@ struct FwdParams {
   const void* src;          // state at t (storage type), [10][nz][ny][nx]
   void* dst;                // state at t+1
   const uint8_t* mask;      // [nz][ny][nx], 1 = solid, or null
+  const uint32_t* links;    // k_stream_collide_sep with walls: per-site wall links (k_wall_links)
+  const uint8_t* tile_dirty;  // and per-tile flags (k_tile_dirty)
   const void* force_field;  // compute type [3][nz][ny][nx] or null (added to the uniform force)
   double force[3];          // uniform body force
   double omega;             // single-component relaxation rate 1/tau
