@@ -127,14 +127,24 @@ int aligned_by(const lbf_params* p) {
 bool sep_built(const lbf_params* p) {
   return !p->two_component && !p->populations && !(p->lattice == LBF_D3Q27H && p->mask != nullptr);
 }
-constexpr int kSepMinZ = 2;  // shortest z-chunk of the axis-separated kernel
+// z-chunks of the axis-separated kernel: at most kSepMaxZ planes, at least two and no fewer than keep a grid
+// of `tiles` columns within kSepBlocks blocks (one 64-byte partial sum each) where that is possible
+constexpr int kSepMaxZ = 96;
+constexpr long long kSepBlocks = 1 << 16;
+int sep_min_z(int nz, long long tiles) {
+  int z = std::min(2, nz);
+  while (z < std::min(kSepMaxZ, nz) && tiles * ((nz + z - 1) / z) > kSepBlocks) ++z;
+  return z;
+}
 // tiles of its largest grid, over both tile heights (walls may add the masked kernel's rows)
 long long sep_max_tiles(const lbf_params* p) {
   const int bytes = int(storage_bytes(p->storage)), Q = p->lattice == LBF_D3Q19 ? 19 : 27;
   const bool high = p->lattice == LBF_D3Q27H;
   const int ty = std::min(sep_config(Q, bytes, high, false).ty, sep_config(Q, bytes, high, true).ty);
-  const int zc = std::min(kSepMinZ, p->nz);
-  return (long long)grid_x(p->nx, 32 * sep_vx(bytes)) * grid_y(p->ny, ty) * ((p->nz + zc - 1) / zc);
+  const long long tiles = (long long)grid_x(p->nx, 32 * sep_vx(bytes)) * grid_y(p->ny, ty);
+  // fewer columns (the taller tile, the rows of a split) may be cut into more chunks: up to kSepBlocks
+  const int zc = sep_min_z(p->nz, tiles);
+  return std::max(tiles * ((p->nz + zc - 1) / zc), std::min(kSepBlocks, tiles * ((p->nz + 1) / 2)));
 }
 
 bool make_layout(const lbf_params* p, Layout* L) {
@@ -553,12 +563,13 @@ lbf_status encode_row_map(const lbf_ctx* c, const void* base, CUtensorMap* out, 
 // walls of a split step the chunks leave at least two waves (min_waves): those CTAs hold SMs as well
 // (200 x 163 x 187 BF16: 24-plane chunks 55.8, 47-plane chunks, one wave, 43.2).
 int choose_zchunk_sep(int nz, long long tiles, double resident, double min_waves) {
-  int zc = nz;
+  const int zmin = sep_min_z(nz, tiles);
+  int zc = std::min(nz, kSepMaxZ);
   double best = 1e30;
   for (int chunks = 1; chunks <= nz; ++chunks) {
     const int z = (nz + chunks - 1) / chunks;
-    if (z < std::min(kSepMinZ, nz)) break;
-    if (z > 96) continue;
+    if (z < zmin) break;
+    if (z > kSepMaxZ) continue;
     const long long nchunks = (nz + z - 1) / z;
     const double waves = double(tiles * nchunks) / resident;
     // many waves run into one another: the last one costs half of itself on average
@@ -761,7 +772,7 @@ lbf_status setup_sep(lbf_ctx* c, const lbf_params* p, const Layout& L, int sms, 
   c->sep.zchunk = choose_zchunk_sep(c->nz, tiles, double(sms) * std::max(resident, 1), c->sep_split ? 2.0 : 1.0);
   if (const char* e = std::getenv("LBF_ZCHUNK")) {
     const int v = std::atoi(e);
-    if (v >= 1) c->sep.zchunk = std::min(c->nz, std::max(std::min(kSepMinZ, c->nz), v));
+    if (v >= 1) c->sep.zchunk = std::min(c->nz, std::max(sep_min_z(c->nz, tiles), v));
   }
   c->sep.grid = dim3(grid_x(c->nx, k.xout), grid_y(c->sep.y_rows, k.by), (c->nz + c->sep.zchunk - 1) / c->sep.zchunk);
   const long long blocks = (long long)c->sep.grid.x * c->sep.grid.y * c->sep.grid.z +
