@@ -339,20 +339,20 @@ unsigned blocks_for(long long n, int threads) {
 }
 
 template <class Tin, class S>
-void launch_encode(const void* src, long long stride, long long site0, long long count, void* dst, long long N, Scales sc,
-                   cudaStream_t st) {
+void launch_encode(const void* src, long long stride, long long site0, long long count, void* dst, void* dst2, long long N,
+                   Scales sc, cudaStream_t st) {
   k_encode<Tin, S><<<blocks_for(count, 256), 256, 0, st>>>(static_cast<const Tin*>(src), stride, site0, count,
-                                                           static_cast<S*>(dst), N, sc);
+                                                           static_cast<S*>(dst), static_cast<S*>(dst2), N, sc);
 }
 
 template <class Tin>
-void encode_dispatch(int storage, const void* src, long long stride, long long site0, long long count, void* dst,
+void encode_dispatch(int storage, const void* src, long long stride, long long site0, long long count, void* dst, void* dst2,
                      long long N, Scales sc, cudaStream_t st) {
   switch (storage) {
-    case LBF_F64: launch_encode<Tin, double>(src, stride, site0, count, dst, N, sc, st); break;
-    case LBF_F32: launch_encode<Tin, float>(src, stride, site0, count, dst, N, sc, st); break;
-    case LBF_F16: launch_encode<Tin, __half>(src, stride, site0, count, dst, N, sc, st); break;
-    case LBF_BF16: launch_encode<Tin, __nv_bfloat16>(src, stride, site0, count, dst, N, sc, st); break;
+    case LBF_F64: launch_encode<Tin, double>(src, stride, site0, count, dst, dst2, N, sc, st); break;
+    case LBF_F32: launch_encode<Tin, float>(src, stride, site0, count, dst, dst2, N, sc, st); break;
+    case LBF_F16: launch_encode<Tin, __half>(src, stride, site0, count, dst, dst2, N, sc, st); break;
+    case LBF_BF16: launch_encode<Tin, __nv_bfloat16>(src, stride, site0, count, dst, dst2, N, sc, st); break;
   }
 }
 
@@ -1276,20 +1276,25 @@ lbf_status lbf_set_moments(lbf_ctx* c, const void* src, int dt, const void* phi)
     set_scales(c, m);
   }
   void* enc_dst = c->pops ? c->mom : c->state[0];  // populations are built from the moments below
+  // a step writes every fluid site of its destination: the second buffer needs the solid sites only. Pageable
+  // host sources of full width pass through it, so it is filled from the first one afterwards
+  const bool both = c->has_mask && !c->pops;
+  const bool through_second = !dev && mapped_host_pointer(src) == nullptr && !c->pops && storage_bytes(c->storage) >= eb;
+  void* enc_dst2 = both && !through_second ? c->state[1] : nullptr;
   if (dev) {
-    if (dt == LBF_F64) encode_dispatch<double>(c->storage, src, N, 0, N, enc_dst, N, c->sc, s);
-    else encode_dispatch<float>(c->storage, src, N, 0, N, enc_dst, N, c->sc, s);
+    if (dt == LBF_F64) encode_dispatch<double>(c->storage, src, N, 0, N, enc_dst, enc_dst2, N, c->sc, s);
+    else encode_dispatch<float>(c->storage, src, N, 0, N, enc_dst, enc_dst2, N, c->sc, s);
     LBF_CUDA(cudaGetLastError());
   } else if (const void* mapped = mapped_host_pointer(src)) {
     // pinned host memory: the encode pass reads it in place over the host link (one pass)
-    if (dt == LBF_F64) encode_dispatch<double>(c->storage, mapped, N, 0, N, enc_dst, N, c->sc, s);
-    else encode_dispatch<float>(c->storage, mapped, N, 0, N, enc_dst, N, c->sc, s);
+    if (dt == LBF_F64) encode_dispatch<double>(c->storage, mapped, N, 0, N, enc_dst, enc_dst2, N, c->sc, s);
+    else encode_dispatch<float>(c->storage, mapped, N, 0, N, enc_dst, enc_dst2, N, c->sc, s);
     LBF_CUDA(cudaGetLastError());
   } else if (!c->pops && storage_bytes(c->storage) >= eb) {
     // the second state buffer holds the whole public state: one host copy, then one encode pass
     LBF_CUDA(cudaMemcpyAsync(c->state[1], src, size_t(10) * N * eb, cudaMemcpyHostToDevice, s));
-    if (dt == LBF_F64) encode_dispatch<double>(c->storage, c->state[1], N, 0, N, enc_dst, N, c->sc, s);
-    else encode_dispatch<float>(c->storage, c->state[1], N, 0, N, enc_dst, N, c->sc, s);
+    if (dt == LBF_F64) encode_dispatch<double>(c->storage, c->state[1], N, 0, N, enc_dst, enc_dst2, N, c->sc, s);
+    else encode_dispatch<float>(c->storage, c->state[1], N, 0, N, enc_dst, enc_dst2, N, c->sc, s);
     LBF_CUDA(cudaGetLastError());
   } else {
     const long long chunk = std::max<long long>(1, (long long)(c->lay.staging_bytes / (10 * eb)));
@@ -1298,8 +1303,8 @@ lbf_status lbf_set_moments(lbf_ctx* c, const void* src, int dt, const void* phi)
       const long long cnt = std::min(chunk, N - s0);
       for (int k = 0; k < 10; ++k)
         LBF_CUDA(cudaMemcpyAsync(c->staging + k * cnt * eb, h + (k * N + s0) * eb, cnt * eb, cudaMemcpyHostToDevice, s));
-      if (dt == LBF_F64) encode_dispatch<double>(c->storage, c->staging, cnt, s0, cnt, enc_dst, N, c->sc, s);
-      else encode_dispatch<float>(c->storage, c->staging, cnt, s0, cnt, enc_dst, N, c->sc, s);
+      if (dt == LBF_F64) encode_dispatch<double>(c->storage, c->staging, cnt, s0, cnt, enc_dst, enc_dst2, N, c->sc, s);
+      else encode_dispatch<float>(c->storage, c->staging, cnt, s0, cnt, enc_dst, enc_dst2, N, c->sc, s);
       LBF_CUDA(cudaGetLastError());
     }
   }
@@ -1308,7 +1313,8 @@ lbf_status lbf_set_moments(lbf_ctx* c, const void* src, int dt, const void* phi)
     void* args[] = {&pp};
     LBF_CUDA(cudaLaunchKernel(c->popk.init, c->pop_grid, dim3(kPopThreads), args, 0, s));
   }
-  LBF_CUDA(cudaMemcpyAsync(c->state[1], c->state[0], lbf_state_bytes(c), cudaMemcpyDeviceToDevice, s));
+  if (c->pops || (both && through_second))
+    LBF_CUDA(cudaMemcpyAsync(c->state[1], c->state[0], lbf_state_bytes(c), cudaMemcpyDeviceToDevice, s));
   c->cur = 0;
   c->pcur = 0;
   if (c->two) {
@@ -1508,7 +1514,8 @@ lbf_status lbf_copy_state(lbf_ctx* c, void* dst) {
 lbf_status lbf_load_state(lbf_ctx* c, const void* src) {
   if (c == nullptr || src == nullptr) return fail(LBF_EINVAL, "NULL argument");
   LBF_CUDA(cudaMemcpyAsync(c->state[c->cur], src, lbf_state_bytes(c), cudaMemcpyDeviceToDevice, c->stream));
-  LBF_CUDA(cudaMemcpyAsync(c->state[1 - c->cur], src, lbf_state_bytes(c), cudaMemcpyDeviceToDevice, c->stream));
+  if (c->has_mask || c->pops)  // the solid sites of the other buffer (a step writes every fluid one)
+    LBF_CUDA(cudaMemcpyAsync(c->state[1 - c->cur], src, lbf_state_bytes(c), cudaMemcpyDeviceToDevice, c->stream));
   c->sums_valid = false;
   return LBF_OK;
 }
