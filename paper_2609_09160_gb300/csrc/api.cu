@@ -123,9 +123,11 @@ int aligned_by(const lbf_params* p) {
                  p->lattice == LBF_D3Q27H);
 }
 
-// the axis-separated kernel is built for a single component, except D3Q27h with walls
+// the axis-separated kernel is built for a single component, except D3Q27h with walls, and for two
+// components on D3Q19 with FP32 storage
 bool sep_built(const lbf_params* p) {
-  return !p->two_component && !p->populations && !(p->lattice == LBF_D3Q27H && p->mask != nullptr);
+  if (p->two_component) return p->lattice == LBF_D3Q19 && p->storage == LBF_F32;
+  return !p->populations && !(p->lattice == LBF_D3Q27H && p->mask != nullptr);
 }
 // z-chunks of the axis-separated kernel: at most kSepMaxZ planes, at least two and no fewer than keep a grid
 // of `tiles` columns within kSepBlocks blocks (one 64-byte partial sum each) where that is possible
@@ -140,7 +142,8 @@ int sep_min_z(int nz, long long tiles) {
 long long sep_max_tiles(const lbf_params* p) {
   const int bytes = int(storage_bytes(p->storage)), Q = p->lattice == LBF_D3Q19 ? 19 : 27;
   const bool high = p->lattice == LBF_D3Q27H;
-  const int ty = std::min(sep_config(Q, bytes, high, false).ty, sep_config(Q, bytes, high, true).ty);
+  const int ty = p->two_component ? sep_config(Q, bytes, high, false, true).ty
+                                  : std::min(sep_config(Q, bytes, high, false).ty, sep_config(Q, bytes, high, true).ty);
   const long long tiles = (long long)grid_x(p->nx, 32 * sep_vx(bytes)) * grid_y(p->ny, ty);
   // fewer columns (the taller tile, the rows of a split) may be cut into more chunks: up to kSepBlocks
   const int zc = sep_min_z(p->nz, tiles);
@@ -231,7 +234,7 @@ struct lbf_ctx {
   unsigned char* staging;
   Scales sc;
   cudaStream_t stream;
-  int zchunk;
+  int zchunk, zchunk_phase;
   dim3 fgrid, agrid;
   KernelInfo fwd, adj;
   KernelInfo fwd_direct;  // the same step loading every site directly (sources TMA cannot read)
@@ -406,14 +409,15 @@ PhaseParams phase_params(const lbf_ctx* c) {
   pp.drho = c->prm.rho_h - c->prm.rho_l;
   pp.mask = c->mask_d;
   pp.sc = c->sc;
-  pp.zchunk = c->zchunk;
+  pp.zchunk = c->zchunk_phase;
   return pp;
 }
 
 // phase-field kernels: the fused step's x-y tiles (30 x kPhaseRows outputs), z-chunks of zchunk
 dim3 phase_block() { return dim3(32, kPhaseRows + 2, 1); }
 dim3 phase_grid(const lbf_ctx* c) {
-  return dim3((c->nx + 29) / 30, (c->ny + kPhaseRows - 1) / kPhaseRows, (c->nz + c->zchunk - 1) / c->zchunk);
+  return dim3((c->nx + 29) / 30, (c->ny + kPhaseRows - 1) / kPhaseRows,
+              (c->nz + c->zchunk_phase - 1) / c->zchunk_phase);
 }
 
 template <class T>
@@ -741,11 +745,16 @@ lbf_status setup_sep(lbf_ctx* c, const lbf_params* p, const Layout& L, int sms, 
   const bool small = kname == "sepsmall" || (kname != "sep" && c->N < (1LL << 20));
   const bool rows_tma = tma_eligible(c->storage, c->nx) && c->nx >= 32 * sep_vx(int(storage_bytes(c->storage)));
   // large lattices whose rows TMA cannot take: the 30-column kernel (333 x 250 x 189: 37.9 against 33.0)
-  if (!rows_tma && !small && !forced) return LBF_OK;
+  if (!rows_tma && !small && !forced && !c->two) return LBF_OK;
   bool walls = c->has_mask;
   c->sep.y_begin = 0;
   c->sep.y_rows = c->ny;
-  if (walls && kname.empty() && !small) {
+  const int two = c->two ? (c->contrast ? 2 : 1) : 0;
+  auto kernel = [&](bool tma) {
+    return two ? sep_two_kernel_for(c->Q, c->storage, walls, two, tma)
+               : sep_kernel_for(c->Q, c->storage, walls, field, tma, nearest, small);
+  };
+  if (walls && kname.empty() && !small && !two) {
     const KernelInfo k = sep_kernel_for(c->Q, c->storage, false, field, false, nearest, small);
     int begin = 0, len = 0;
     if (!clean_band(c, p, k.by, &begin, &len)) return LBF_OK;  // scattered walls: the 30-column kernel
@@ -758,10 +767,10 @@ lbf_status setup_sep(lbf_ctx* c, const lbf_params* p, const Layout& L, int sms, 
     c->zchunk_dirty = std::min(LBF_SPLIT_ZCHUNK, c->nz);
     c->grid_dirty = dim3(grid_x(c->nx, c->fwd.xout), grid_y(c->dirty_rows, c->fwd.by), (c->nz + c->zchunk_dirty - 1) / c->zchunk_dirty);
   }
-  c->sep.async = sep_kernel_for(c->Q, c->storage, walls, field, false, nearest, small);
+  c->sep.async = kernel(false);
   c->sep.tma = KernelInfo{nullptr, 0, 0, 0, 0};
   if (rows_tma)
-    c->sep.tma = sep_kernel_for(c->Q, c->storage, walls, field, true, nearest, small);
+    c->sep.tma = kernel(true);
   lbf_status st;
   if ((st = prepare(c->sep.async)) != LBF_OK || (st = prepare(c->sep.tma)) != LBF_OK) return st;
   const KernelInfo& k = c->sep.tma.fn ? c->sep.tma : c->sep.async;
@@ -1172,6 +1181,10 @@ lbf_status lbf_create(lbf_ctx** out, const lbf_params* params, void* workspace, 
     if (v >= 1) zc = std::max(min_zchunk(c->nz), v);
   }
   c->zchunk = std::min(zc, c->nz);
+  // phase-field kernels: short chunks fill the chip on small lattices and cost the large ones nothing (the
+  // restaged planes hit L2). us a step at 6 / 11 / 15 planes: droplet 128^3 113.0 / 113.7 / 114.5, layered
+  // 512 x 1024 x 8 282.9 / 284.2 / 285.2, 96 x 90 x 70 59.0 / 63.7 / 68.7
+  c->zchunk_phase = std::min(6, c->nz);
   c->fgrid = dim3(grid_x(c->nx, c->fwd.xout), grid_y(c->ny, c->fwd.by), (c->nz + c->zchunk - 1) / c->zchunk);
   c->agrid = c->adj.fn ? dim3(grid_x(c->nx), grid_y(c->ny, c->adj.by), (c->nz + c->zchunk - 1) / c->zchunk) : dim3(1, 1, 1);
   if (c->tma) {

@@ -179,7 +179,9 @@ __global__ void k_reduce_final(const double* __restrict__ partials, long long nb
 // systematic change of sum(phi) into every step. The kernels march along z with the same x-y tiles as
 // the fused step (32 columns of which 30 are outputs, BY + 2 rows): every thread keeps three planes
 // of its own column in registers and applies the z filters there, one shared-memory plane holds the
-// z-filtered values, and the outputs apply the x-y filters from it.
+// z-filtered values, and the outputs apply the x-y filters from it. What bounds them is latency (128^3: one
+// wave of CTAs, 6 per SM, marching 17 planes): the plane's shared memory is double, so a plane has one
+// barrier.
 struct PhaseParams {
   int nx, ny, nz;
   long long N;
@@ -244,64 +246,66 @@ struct PhaseColumn {
 // With walls, u is taken as 0 at solid sites and phi is not advanced there (it keeps its value),
 // so a wall in contact with one bulk phase exchanges no phi.
 template <class S, class T>
-__global__ void __launch_bounds__(PhaseTile<T>::SITES) k_phase_advance(const S* __restrict__ st,
+__global__ void __launch_bounds__(PhaseTile<T>::SITES, sizeof(T) == 4 ? 6 : 1) k_phase_advance(const S* __restrict__ st,
                                                                        const T* __restrict__ phi,
                                                                        const T* __restrict__ G,
                                                                        T* __restrict__ phi_new, PhaseParams p) {
   using PT = PhaseTile<T>;
-  __shared__ T sm[5][PT::SITES];  // phi, L_z phi, A_z V_x, A_z V_y, D_z V_z of the current plane
+  __shared__ T sm[2][5][PT::SITES];  // phi, L_z phi, A_z V_x, A_z V_y, D_z V_z of the current plane
   const PhaseColumn c(p);
   const int me = threadIdx.y * 32 + threadIdx.x;
   const long long N = p.N, plane = (long long)p.nx * p.ny;
   const T lam = T(p.lambda), dif6 = T(6) * T(p.D);
   // planes z-1, z, z+1 of this column: phi and V
   T f[3], vx[3], vy[3], vz[3];
-  // raw values of the plane after those (prefetched)
-  T rph, rux, ruy, ruz, rgx, rgy, rgz;
-  auto fetch = [&](int zp) {
+  struct Raw {  // stored values of a plane
+    T ph, ux, uy, uz, gx, gy, gz;
+  };
+  auto fetch = [&](int zp, Raw& r) {
     const long long s = (long long)wrap(zp, p.nz) * plane + c.col;  // zp in [-1, nz]
-    rph = phi[s];
+    r.ph = phi[s];
     if constexpr (Codec<S>::scaled) {
-      rux = T(Codec<S>::load(st + N + s) * p.sc.dec[1]);
-      ruy = T(Codec<S>::load(st + 2 * N + s) * p.sc.dec[1]);
-      ruz = T(Codec<S>::load(st + 3 * N + s) * p.sc.dec[1]);
+      r.ux = T(Codec<S>::load(st + N + s) * p.sc.dec[1]);
+      r.uy = T(Codec<S>::load(st + 2 * N + s) * p.sc.dec[1]);
+      r.uz = T(Codec<S>::load(st + 3 * N + s) * p.sc.dec[1]);
     } else {
-      rux = st[N + s];
-      ruy = st[2 * N + s];
-      ruz = st[3 * N + s];
+      r.ux = st[N + s];
+      r.uy = st[2 * N + s];
+      r.uz = st[3 * N + s];
     }
-    rgx = G[s];
-    rgy = G[N + s];
-    rgz = G[2 * N + s];
-    if (p.mask != nullptr && p.mask[s]) rux = ruy = ruz = T(0);
+    r.gx = G[s];
+    r.gy = G[N + s];
+    r.gz = G[2 * N + s];
+    if (p.mask != nullptr && p.mask[s]) r.ux = r.uy = r.uz = T(0);
   };
-  auto take = [&](int k) {
-    f[k] = rph;
-    vx[k] = rph * rux + lam * rgx;
-    vy[k] = rph * ruy + lam * rgy;
-    vz[k] = rph * ruz + lam * rgz;
+  auto take = [&](int k, const Raw& r) {
+    f[k] = r.ph;
+    vx[k] = r.ph * r.ux + lam * r.gx;
+    vy[k] = r.ph * r.uy + lam * r.gy;
+    vz[k] = r.ph * r.uz + lam * r.gz;
   };
-  fetch(c.z0 - 1);
-  take(0);
-  fetch(c.z0);
-  take(1);
-  fetch(c.z0 + 1);
+  Raw r0, r1;
+  fetch(c.z0 - 1, r0);
+  fetch(c.z0, r1);
+  take(0, r0);
+  fetch(c.z0 + 1, r0);
+  take(1, r1);
   for (int z = c.z0; z < c.z1; ++z) {
-    take(2);
-    if (z + 2 <= c.z1) fetch(z + 2);  // in flight during this plane
-    sm[0][me] = f[1];
-    sm[1][me] = PT::A1 * ((f[0] - f[1]) + (f[2] - f[1]));
-    sm[2][me] = PT::A0 * vx[1] + PT::A1 * (vx[0] + vx[2]);
-    sm[3][me] = PT::A0 * vy[1] + PT::A1 * (vy[0] + vy[2]);
-    sm[4][me] = PT::A1 * (vz[2] - vz[0]);
+    take(2, r0);
+    if (z + 2 <= c.z1) fetch(z + 2, r0);  // in flight during this plane
+    T(*const b)[PT::SITES] = sm[(z - c.z0) & 1];
+    b[0][me] = f[1];
+    b[1][me] = PT::A1 * ((f[0] - f[1]) + (f[2] - f[1]));
+    b[2][me] = PT::A0 * vx[1] + PT::A1 * (vx[0] + vx[2]);
+    b[3][me] = PT::A0 * vy[1] + PT::A1 * (vy[0] + vy[2]);
+    b[4][me] = PT::A1 * (vz[2] - vz[0]);
     __syncthreads();
     if (c.out) {
-      const T div = PT::dxay(sm[2] + me) + PT::dyax(sm[3] + me) + PT::axay(sm[4] + me);
-      const T lap = PT::lap_xy(sm[0] + me) + PT::axay(sm[1] + me);
+      const T div = PT::dxay(b[2] + me) + PT::dyax(b[3] + me) + PT::axay(b[4] + me);
+      const T lap = PT::lap_xy(b[0] + me) + PT::axay(b[1] + me);
       const long long s = (long long)z * plane + c.col;
       phi_new[s] = (p.mask != nullptr && p.mask[s]) ? f[1] : f[1] - T(3) * div + dif6 * lap;
     }
-    __syncthreads();
     f[0] = f[1];
     f[1] = f[2];
     vx[0] = vx[1];
@@ -319,11 +323,11 @@ __global__ void __launch_bounds__(PhaseTile<T>::SITES) k_phase_advance(const S* 
 // With a density contrast grad phi is also written (gphi, else null): the fused step forms the
 // pressure and viscous-gradient forces from it and the raw moments of the new state.
 template <class T>
-__global__ void __launch_bounds__(PhaseTile<T>::SITES) k_phase_forces(const T* __restrict__ phi,
+__global__ void __launch_bounds__(PhaseTile<T>::SITES, sizeof(T) == 4 ? 6 : 1) k_phase_forces(const T* __restrict__ phi,
                                                                       T* __restrict__ F, T* __restrict__ G,
                                                                       T* __restrict__ gphi, PhaseParams p) {
   using PT = PhaseTile<T>;
-  __shared__ T sm[4][PT::SITES];  // A_z phi, D_z phi, phi, L_z phi of the current plane
+  __shared__ T sm[2][4][PT::SITES];  // A_z phi, D_z phi, phi, L_z phi of the current plane
   const PhaseColumn c(p);
   const int me = threadIdx.y * 32 + threadIdx.x;
   const long long N = p.N, plane = (long long)p.nx * p.ny;
@@ -332,18 +336,23 @@ __global__ void __launch_bounds__(PhaseTile<T>::SITES) k_phase_forces(const T* _
   const T a0 = T(p.accel[0]), a1 = T(p.accel[1]), a2 = T(p.accel[2]);
   const T rl = T(p.rho_l), dr = T(p.drho);
   auto fetch = [&](int zp) { return phi[(long long)wrap(zp, p.nz) * plane + c.col]; };  // zp in [-1, nz]
-  T f0 = fetch(c.z0 - 1), f1 = fetch(c.z0), f2, nxt = fetch(c.z0 + 1);
+  T f0 = fetch(c.z0 - 1), f1 = fetch(c.z0), f2, n0 = fetch(c.z0 + 1), n1 = T(0), n2 = T(0);
+  if (c.z0 + 2 <= c.z1) n1 = fetch(c.z0 + 2);
+  if (c.z0 + 3 <= c.z1) n2 = fetch(c.z0 + 3);
   for (int z = c.z0; z < c.z1; ++z) {
-    f2 = nxt;
-    if (z + 2 <= c.z1) nxt = fetch(z + 2);
-    sm[0][me] = PT::A0 * f1 + PT::A1 * (f0 + f2);
-    sm[1][me] = PT::A1 * (f2 - f0);
-    sm[2][me] = f1;
-    sm[3][me] = PT::A1 * ((f0 - f1) + (f2 - f1));
+    f2 = n0;
+    n0 = n1;
+    n1 = n2;
+    if (z + 4 <= c.z1) n2 = fetch(z + 4);
+    T(*const b)[PT::SITES] = sm[(z - c.z0) & 1];
+    b[0][me] = PT::A0 * f1 + PT::A1 * (f0 + f2);
+    b[1][me] = PT::A1 * (f2 - f0);
+    b[2][me] = f1;
+    b[3][me] = PT::A1 * ((f0 - f1) + (f2 - f1));
     __syncthreads();
     if (c.out) {
-      const T gx = T(3) * PT::dxay(sm[0] + me), gy = T(3) * PT::dyax(sm[0] + me), gz = T(3) * PT::axay(sm[1] + me);
-      const T lap = T(6) * (PT::lap_xy(sm[2] + me) + PT::axay(sm[3] + me));
+      const T gx = T(3) * PT::dxay(b[0] + me), gy = T(3) * PT::dyax(b[0] + me), gz = T(3) * PT::axay(b[1] + me);
+      const T lap = T(6) * (PT::lap_xy(b[2] + me) + PT::axay(b[3] + me));
       const T mu = beta4 * f1 * (f1 - T(1)) * (f1 - T(0.5)) - kappa * lap;
       const long long s = (long long)z * plane + c.col;
       const T rho = rl + f1 * dr;
@@ -362,7 +371,6 @@ __global__ void __launch_bounds__(PhaseTile<T>::SITES) k_phase_forces(const T* _
       G[N + s] = cc * gy;
       G[2 * N + s] = cc * gz;
     }
-    __syncthreads();
     f0 = f1;
     f1 = f2;
   }

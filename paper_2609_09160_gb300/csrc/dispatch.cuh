@@ -129,13 +129,13 @@ KernelInfo aligned_kernel_ls(bool mask, bool field, bool nearest) {
 // the axis-separated kernel (single component). fn == nullptr for D3Q27h with walls, which is not
 // built (its wall populations need the full basis). small: the tile for lattices that leave most of the
 // chip idle; tma: rows by TMA, else by cp.async (16-bit storage: nx must be even)
-template <class L, class S, bool SMALL, bool TMA, bool MASK, bool FF, bool RN>
+template <class L, class S, bool SMALL, bool TMA, bool MASK, bool FF, bool RN, int TWO = 0>
 KernelInfo sep_info() {
-  constexpr SepConfig C = sep_config(L::Q, int(sizeof(S)), L::HIGH, SMALL);
+  constexpr SepConfig C = sep_config(L::Q, int(sizeof(S)), L::HIGH, SMALL, TWO != 0);
   constexpr int VX = sep_vx(int(sizeof(S)));
   using G = SepTile<L, S, VX, C.ty, C.rp>;
   KernelInfo k;
-  k.fn = reinterpret_cast<const void*>(&k_stream_collide_sep<L, S, SMALL, TMA, MASK, FF, RN>);
+  k.fn = reinterpret_cast<const void*>(&k_stream_collide_sep<L, S, SMALL, TMA, MASK, FF, RN, TWO>);
   k.smem = sep_smem_bytes<L, S, VX, C.ty, C.rp, C.stages, MASK>();
   k.threads = G::THREADS;
   k.by = C.ty;
@@ -171,6 +171,22 @@ KernelInfo sep_kernel_ls(bool mask, bool field, bool tma, bool nearest, bool sma
   }
 }
 
+// the axis-separated kernel with two components (two: 1 equal densities, 2 a density contrast): D3Q19 FP32
+template <class L, class S>
+KernelInfo sep_two_ls(bool mask, int two, bool tma) {
+  if constexpr (L::Q == 19 && std::is_same<S, float>::value) {
+    if (two == 2) {
+      if (mask) return tma ? sep_info<L, S, false, true, true, false, false, 2>() : sep_info<L, S, false, false, true, false, false, 2>();
+      return tma ? sep_info<L, S, false, true, false, false, false, 2>() : sep_info<L, S, false, false, false, false, false, 2>();
+    }
+    if (mask) return tma ? sep_info<L, S, false, true, true, false, false, 1>() : sep_info<L, S, false, false, true, false, false, 1>();
+    return tma ? sep_info<L, S, false, true, false, false, false, 1>() : sep_info<L, S, false, false, false, false, false, 1>();
+  } else {
+    (void)mask, (void)two, (void)tma;
+    return KernelInfo{nullptr, 0, 0, 0, 0};
+  }
+}
+
 // population-form reference kernels of lattice L, storage S (FP32/FP64 only; nulls otherwise)
 struct PopKernels {
   const void* step;     // k_pop_step
@@ -202,6 +218,7 @@ PopKernels pop_kernels_ls(bool mask, bool field) {
   KernelInfo forward_kernel_q##q##_s##s(bool mask, int two, bool field, bool tma, bool nearest); \
   KernelInfo aligned_kernel_q##q##_s##s(bool mask, bool field, bool nearest);                    \
   KernelInfo sep_kernel_q##q##_s##s(bool mask, bool field, bool tma, bool nearest, bool small);  \
+  KernelInfo sep_two_q##q##_s##s(bool mask, int two, bool tma);                                  \
   PopKernels pop_kernels_q##q##_s##s(bool mask, bool field);                                        \
   KernelInfo adjoint_kernel_q##q##_s##s(bool mask);
 LBF_DECLARE_TU(19, 0)
@@ -280,6 +297,11 @@ inline KernelInfo sep_kernel_for(int lattice, int storage, bool mask, bool field
     LBF_SEP_CASE(127)
   }
 #undef LBF_SEP_CASE
+  return KernelInfo{nullptr, 0, 0, 0, 0};
+}
+
+inline KernelInfo sep_two_kernel_for(int lattice, int storage, bool mask, int two, bool tma) {
+  if (lattice == 19 && storage == ST_F32) return sep_two_q19_s1(mask, two, tma);
   return KernelInfo{nullptr, 0, 0, 0, 0};
 }
 

@@ -48,6 +48,10 @@ KernelInfo LBF_CAT(sep_kernel_q, LBF_TU_LATTICE, _s, LBF_TU_STORAGE)(bool mask, 
   return sep_kernel_ls<TuL, TuS>(mask, field, tma, nearest, small);
 }
 
+KernelInfo LBF_CAT(sep_two_q, LBF_TU_LATTICE, _s, LBF_TU_STORAGE)(bool mask, int two, bool tma) {
+  return sep_two_ls<TuL, TuS>(mask, two, tma);
+}
+
 PopKernels LBF_CAT(pop_kernels_q, LBF_TU_LATTICE, _s, LBF_TU_STORAGE)(bool mask, bool field) {
 #if LBF_TU_LATTICE == 127
   (void)mask;

@@ -48,6 +48,9 @@
 //     CTA per SM with 5 stages of 8 rows (72) over two of 6 rows with 4 (67).
 //   * outputs leave as TMA boxes from the stage rows just read: 62.6 -> 68.6 (FP32 256^3) against per-thread
 //     stores, which queue in front of the other warps' shared-memory accesses.
+//   * two components (TWO): the forces and phase field of the source and of the output sites are loaded as
+//     pairs one plane ahead: droplet 128^3 72 -> 56 us a launch against scalar loads (83 before), layered
+//     contrast flow 205 -> 175; 8 warps of 126 registers, two CTAs per SM (6 warps 118, here 115 us a step).
 //   * rows 0 and TY + 1 and the halo columns on two warps of their own: the warp that carried both took
 //     2100 of the 2120 cycles of a plane while the output rows took 1500.
 
@@ -180,8 +183,12 @@ struct SepConfig {
 #ifndef LBF_SEP_CFG_SMALL
 #define LBF_SEP_CFG_SMALL 40412
 #endif
-constexpr SepConfig sep_config(int Q, int bytes, bool high, bool small) {
-  const int c = bytes == 8   ? LBF_SEP_CFG_F64
+#ifndef LBF_SEP_CFG_TWO
+#define LBF_SEP_CFG_TWO 40612
+#endif
+constexpr SepConfig sep_config(int Q, int bytes, bool high, bool small, bool two = false) {
+  const int c = two          ? LBF_SEP_CFG_TWO
+                : bytes == 8 ? LBF_SEP_CFG_F64
                 : small      ? LBF_SEP_CFG_SMALL
                 : Q == 19    ? (bytes == 4 ? LBF_SEP_CFG_Q19 : LBF_SEP_CFG_Q19_16)
                 : high       ? (bytes == 4 ? LBF_SEP_CFG_Q27H : LBF_SEP_CFG_Q27H_16)
@@ -234,7 +241,8 @@ __device__ __forceinline__ float2 ld_pair(const S* p) {
 
 // ---- coefficients -------------------------------------------------------------------------------
 // f_c / w_c = q0 + b.c + exx cx^2 + ... + exy cx cy + ... from the moments, F = 2 rho h the force (rho = 1)
-// and keep = 1 - omega (times the decode factor of N): with P2 = u u + keep N + u h + h u,
+// and k1 = 1 - omega (times the decode factor of N; F / rho in the place of F with two components): with
+// P2 = u u + k1 N + u h + h u,
 //   q0 = p* - (3/2) tr P2, b = 3 (u + h), e_aa = (9/2) P2_aa, e_ab = 9 P2_ab.
 // Every constant is exact in FP32: p* and u pass through a step with a factor of one, and a factor 1/3
 // rounded here would grow by 3e-8 a step.
@@ -243,8 +251,8 @@ struct SepCoef {
   V q0, bx, by, bz, exx, eyy, ezz, exy, exz, eyz;
 };
 template <class T, class V>
-__device__ __forceinline__ SepCoef<V> sep_coef(const V (&m)[10], const V (&F)[3], T keep) {
-  const V k1 = v_set<V>(keep), k9 = v_set<V>(T(9) * keep), three = v_set<V>(T(3)), nine = v_set<V>(T(9));
+__device__ __forceinline__ SepCoef<V> sep_coef(const V (&m)[10], const V (&F)[3], V k1) {
+  const V k9 = v_mul(k1, v_set<V>(T(9))), three = v_set<V>(T(3)), nine = v_set<V>(T(9));
   const V f15 = v_set<V>(T(1.5)), f45 = v_set<V>(T(4.5));
   const V ux = m[1], uy = m[2], uz = m[3];
   const V gx = v_mul(F[0], f45), gy = v_mul(F[1], f45), gz = v_mul(F[2], f45);  // 9 h
@@ -333,13 +341,13 @@ __device__ __forceinline__ void cta_barrier() {
   asm volatile("barrier.cta.sync 1, %0;" ::"n"(THREADS) : "memory");
 }
 
-template <class L, class S, bool SMALL, bool TMA, bool MASK, bool FF, bool RN>
-__global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH, SMALL).ty /
-                                            sep_config(L::Q, int(sizeof(S)), L::HIGH, SMALL).rp + 2),
-                                  sep_config(L::Q, int(sizeof(S)), L::HIGH, SMALL).minb)
+template <class L, class S, bool SMALL, bool TMA, bool MASK, bool FF, bool RN, int TWO = 0>
+__global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH, SMALL, TWO != 0).ty /
+                                            sep_config(L::Q, int(sizeof(S)), L::HIGH, SMALL, TWO != 0).rp + 2),
+                                  sep_config(L::Q, int(sizeof(S)), L::HIGH, SMALL, TWO != 0).minb)
     k_stream_collide_sep(const FwdParams a, const __grid_constant__ CUtensorMap trow,
                          const __grid_constant__ CUtensorMap ttile, const __grid_constant__ CUtensorMap tout) {
-  constexpr SepConfig CFG = sep_config(L::Q, int(sizeof(S)), L::HIGH, SMALL);
+  constexpr SepConfig CFG = sep_config(L::Q, int(sizeof(S)), L::HIGH, SMALL, TWO != 0);
   constexpr int VX = sep_vx(int(sizeof(S))), TY = CFG.ty, RP = CFG.rp, STAGES = CFG.stages;
   using G = SepTile<L, S, VX, TY, RP>;
   using T = typename ComputeOf<S>::type;
@@ -392,7 +400,7 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
   // halo columns: side 0 = left (p), 1 = right (m), written one plane ahead, read by the edge lanes
   auto hx_at = [&](int ip, int side, int r) { return hx + ((ip & 1) * 2 + side) * ROWS * NEP + r * NEP; };
 
-  constexpr bool AHEAD = FF || MASK;  // the rows too load something into registers one plane ahead
+  constexpr bool AHEAD = FF || MASK || TWO != 0;  // the rows too load something into registers one plane ahead
 
   // ---- what a thread reads of one plane, for its row's sites or for the halo columns --------------
   struct Site {
@@ -401,8 +409,11 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
     bool needed;    // the row is read by some output
   };
   // what is loaded into registers one plane ahead besides the x-halo values: per-site force, wall links
+  constexpr bool SITEF = FF || TWO != 0;  // a force of its own at every site
+  static_assert(TWO == 0 || (!FF && std::is_same<S, T>::value && !L::HIGH), "two components: FP32 or FP64 storage, no force field");
   struct Extra {
-    T f0[FF ? 3 : 1], f1[FF ? 3 : 1];
+    T f0[SITEF ? 3 : 1], f1[SITEF ? 3 : 1];
+    T p0, p1;  // two components: phi^n
     uint32_t l0, l1;
   };
   auto fetch_values = [&](const Site& t, int ip, S (&v0)[10], S (&v1)[10]) {
@@ -424,6 +435,28 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
         if constexpr (VX == 2) r.f1[k] = __ldg(ffield + k * N + zoff + t.o1);
       }
     }
+    if constexpr (TWO != 0) {
+      const T* Fo = static_cast<const T*>(a.F_old) + zoff;
+      const T* po = static_cast<const T*>(a.phi_old) + zoff;
+      // the library's own arrays: 8-byte aligned pairs where the rows hold whole 16-byte units (TMA)
+      if (TMA && VX == 2 && t.o1 == t.o0 + 1) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const float2 q = __ldg(reinterpret_cast<const float2*>(Fo + k * N + t.o0));
+          r.f0[k] = q.x, r.f1[k] = q.y;
+        }
+        const float2 q = __ldg(reinterpret_cast<const float2*>(po + t.o0));
+        r.p0 = q.x, r.p1 = q.y;
+      } else {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          r.f0[k] = __ldg(Fo + k * N + t.o0);
+          if constexpr (VX == 2) r.f1[k] = __ldg(Fo + k * N + t.o1);
+        }
+        r.p0 = __ldg(po + t.o0);
+        if constexpr (VX == 2) r.p1 = __ldg(po + t.o1);
+      }
+    }
     if constexpr (MASK) {
       if (dirty) {
         r.l0 = __ldg(a.links + zoff + t.o0);
@@ -443,8 +476,37 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
     for (int k = 0; k < 10; ++k)
       m[k] = t.needed ? pack(static_cast<T>(v0[k]), VX == 2 ? static_cast<T>(v1[k]) : T(0)) : zero;
   };
+  // two components: rho(phi) = rho_l + phi drho, nu(phi) = nu_l + phi dnu, 1 - omega = 1 - 1 / (3 nu + 1/2)
+  const T rho_l = pick<T>(a.rho_l, a.rho_l_f), drho = pick<T>(a.rho_h - a.rho_l, a.drho_f);
+  const T nu_l = pick<T>(a.nu_l, a.nu_l_f), dnu = pick<T>(a.nu_h - a.nu_l, a.dnu_f);
+  const T rrho_l = TWO != 0 ? T(1) / rho_l : T(1), keep_l = TWO != 0 ? T(1) - T(1) / (T(3) * nu_l + T(0.5)) : T(0);
+  auto each = [&](V v, auto f) -> V {
+    if constexpr (VX == 2)
+      return make_float2(f(v.x), f(v.y));
+    else
+      return f(v);
+  };
+  auto rrho_of = [&](V phi) -> V {  // 1 / rho
+    if constexpr (TWO == 2)
+      return each(phi, [&](T p) { return T(1) / (rho_l + p * drho); });
+    else
+      return v_set<V>(rrho_l);
+  };
+  auto keep_of = [&](const Extra& r) -> V {
+    if constexpr (TWO != 0) {
+      if (dnu == T(0)) return v_set<V>(keep_l);
+      return each(pack(r.p0, VX == 2 ? r.p1 : T(0)), [&](T p) { return T(1) - T(1) / (T(3) * (nu_l + p * dnu) + T(0.5)); });
+    } else {
+      return v_set<V>(keep);
+    }
+  };
+  // the force at the sites (two components: F / rho, as it enters the collision)
   auto force_of = [&](const Extra& r, V (&F)[3]) {
-    if constexpr (FF) {
+    if constexpr (TWO != 0) {
+      const V rr = rrho_of(pack(r.p0, VX == 2 ? r.p1 : T(0)));
+#pragma unroll
+      for (int k = 0; k < 3; ++k) F[k] = v_mul(pack(r.f0[k], VX == 2 ? r.f1[k] : T(0)), rr);
+    } else if constexpr (FF) {
       F[0] = pack(Fu0 + r.f0[0], VX == 2 ? Fu0 + r.f1[0] : T(0));
       F[1] = pack(Fu1 + r.f0[1], VX == 2 ? Fu1 + r.f1[1] : T(0));
       F[2] = pack(Fu2 + r.f0[2], VX == 2 ? Fu2 + r.f1[2] : T(0));
@@ -490,7 +552,7 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
     force_of(r, F);
     V P[NE], M[NE];
     if constexpr (!L::HIGH) {
-      SepCoef<V> c = sep_coef<T, V>(m, F, keep);
+      SepCoef<V> c = sep_coef<T, V>(m, F, keep_of(r));
       silence(c, r);
       const V az = v_add(c.q0, c.ezz);
       const V tp = v_add(v_add(az, c.bz), c.exx), tm = v_add(v_sub(az, c.bz), c.exx), t0 = v_add(c.q0, c.exx);
@@ -555,7 +617,7 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
     return r;
   };
   auto fetch = [&](RowIn& r, int ip) {
-    if constexpr (FF || MASK) fetch_extra(r.t, ip, r.e);
+    if constexpr (AHEAD) fetch_extra(r.t, ip, r.e);
   };
   // without TMA: every thread copies its own sites into the stage (cp.async, 4 or 8 bytes each) as many
   // planes ahead as TMA would, and waits for its own copies only
@@ -630,7 +692,7 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
     };
     const V two = v_set<V>(T(2)), four = v_set<V>(T(4));
     if constexpr (!L::HIGH) {
-      SepCoef<V> c = sep_coef<T, V>(m, F, keep);
+      SepCoef<V> c = sep_coef<T, V>(m, F, keep_of(in.e));
       silence(c, in.e);
       if constexpr (MASK) {
         if (dirty && outputs) {
@@ -803,7 +865,7 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
     hext.l0 = hext.l1 = 0u;
     auto hfetch = [&](int ip) {
       fetch_values(ht, ip, hraw0, hraw1);
-      if constexpr (FF || MASK) fetch_extra(ht, ip, hext);
+      if constexpr (AHEAD) fetch_extra(ht, ip, hext);
     };
     const int rows = min(ROWS, yrows + 2 - ybl), rs = row_of(min(lane, ROWS - 1));
     // all rows at once where they are consecutive in the lattice, else (y wrap, last rows) one by one:
@@ -869,6 +931,7 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
       V a0, jx, jy, jz, rxx, ryy, rzz, rxy, rxz, ryz;
       V u00, u10, u01, u20, u02, u11;
       V hx, hy, hz;      // half force of the plane below (FF)
+      V n0[TWO != 0 ? 3 : 1], np[1], ng[TWO == 2 ? 3 : 1];  // two components: F^{n+1}, phi^{n+1}, grad phi^{n+1} there
       bool sol0, sol1;   // its solid flags
     };
     RowIn in[RP];
@@ -884,6 +947,29 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
       f.sol0 = f.sol1 = false;
       if constexpr (AHEAD) fetch(in[r], 0);
     }
+    // two components: the correction's inputs of plane ip, loaded when it is taken in, used a plane later
+    auto fetch_new = [&](const RowIn& r, Flight& f, int ip) {
+      if constexpr (TWO != 0) {
+        if (!r.t.needed) return;
+        const long long zoff = (long long)wrap(z0 - 1 + ip, a.nz) * plane;
+        const T* Fn = static_cast<const T*>(a.F_new) + zoff;  // rewritten (TWO = 2) only at the site's own output
+        const T* pn = static_cast<const T*>(a.phi_new) + zoff;
+        auto two_of = [&](const T* q) -> V {
+          if constexpr (VX == 2 && TMA)
+            return *reinterpret_cast<const float2*>(q + r.t.o0);
+          else
+            return pack(q[r.t.o0], VX == 2 ? q[r.t.o1] : T(0));
+        };
+#pragma unroll
+        for (int k = 0; k < 3; ++k) f.n0[k] = two_of(Fn + k * N);
+        f.np[0] = two_of(pn);
+        if constexpr (TWO == 2) {
+          const T* gp = static_cast<const T*>(a.grad_phi) + zoff;
+#pragma unroll
+          for (int k = 0; k < 3; ++k) f.ng[k] = two_of(gp + k * N);
+        }
+      }
+    };
     bool bad = false;
     // whole rows of fluid sites leave as one TMA box from the stage rows the warp has just read
     for (int p = 0; p < STAGES - 1; ++p) {
@@ -975,8 +1061,46 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
           const V vs = v_set<V>(sc), vl = v_set<V>(lack);
           auto scaled = [&](V v) -> V { return v_fma(v, vs, v_mul(v, vl)); };
           const V b0 = scaled(f.a0);
+          const bool own_row = ybl + warp * RP + r < yrows;
+          const bool w0 = own_row && gx >= xb && gx < nx && !f.sol0;
+          const bool w1 = VX == 2 && own_row && gx >= xb && gx + 1 < nx && !f.sol1;
+          const long long zc = (long long)z * plane + in[r].t.o0;
           V hx_, hy_, hz_;
-          if constexpr (FF)
+          if constexpr (TWO != 0) {
+            V Fn[3] = {f.n0[0], f.n0[1], f.n0[2]};
+            if constexpr (TWO == 2) {
+              // density contrast (Sec. 2 force split): the force of the new state adds to F^s + F^b
+              //   F^p = -p* cs2 grad rho and F^nu = -(nu omega / cs2) a*_neq . grad rho,
+              // with p* = a*0 and a*_neq = a*2 - a*1 a*1 the raw moments just streamed in
+              const V jx_ = scaled(f.jx), jy_ = scaled(f.jy), jz_ = scaled(f.jz);
+              const V dr = v_set<V>(drho), gr0 = v_mul(f.ng[0], dr), gr1 = v_mul(f.ng[1], dr), gr2 = v_mul(f.ng[2], dr);
+              const V p3 = v_mul(b0, v_set<V>(T(1) / T(3)));
+              const V qxx = v_nfma(jx_, jx_, v_sub(v_mul(f.rxx, vs), p3));
+              const V qyy = v_nfma(jy_, jy_, v_sub(v_mul(f.ryy, vs), p3));
+              const V qzz = v_nfma(jz_, jz_, v_sub(v_mul(f.rzz, vs), p3));
+              const V qxy = v_nfma(jx_, jy_, v_mul(f.rxy, vs)), qxz = v_nfma(jx_, jz_, v_mul(f.rxz, vs));
+              const V qyz = v_nfma(jy_, jz_, v_mul(f.ryz, vs));
+              const V cnu = each(f.np[0], [&](T p) {
+                const T nu = nu_l + p * dnu;
+                return T(-3) * nu / (T(3) * nu + T(0.5));
+              });
+              Fn[0] = v_add(Fn[0], v_nfma(p3, gr0, v_mul(cnu, v_fma(qxx, gr0, v_fma(qxy, gr1, v_mul(qxz, gr2))))));
+              Fn[1] = v_add(Fn[1], v_nfma(p3, gr1, v_mul(cnu, v_fma(qxy, gr0, v_fma(qyy, gr1, v_mul(qyz, gr2))))));
+              Fn[2] = v_add(Fn[2], v_nfma(p3, gr2, v_mul(cnu, v_fma(qxz, gr0, v_fma(qyz, gr1, v_mul(qzz, gr2))))));
+              T* Fw = static_cast<T*>(a.F_new) + (long long)z * plane;
+#pragma unroll
+              for (int k = 0; k < 3; ++k) {
+                if constexpr (VX == 2) {
+                  if (w0) Fw[k * N + in[r].t.o0] = Fn[k].x;
+                  if (w1) Fw[k * N + in[r].t.o1] = Fn[k].y;
+                } else {
+                  if (w0) Fw[k * N + in[r].t.o0] = Fn[k];
+                }
+              }
+            }
+            const V hr = v_mul(rrho_of(f.np[0]), v_set<V>(T(0.5)));
+            hx_ = v_mul(Fn[0], hr), hy_ = v_mul(Fn[1], hr), hz_ = v_mul(Fn[2], hr);
+          } else if constexpr (FF)
             hx_ = f.hx, hy_ = f.hy, hz_ = f.hz;
           else
             hx_ = v_set<V>(T(0.5) * Fu0), hy_ = v_set<V>(T(0.5) * Fu1), hz_ = v_set<V>(T(0.5) * Fu2);
@@ -992,10 +1116,6 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
           const V nxz = v_nfma(vx, vz, v_fma(f.rxz, vs, v_mul(hx_, hz_)));
           const V nyz = v_nfma(vy, vz, v_fma(f.ryz, vs, v_mul(hy_, hz_)));
           const V uu = v_fma(ux, ux, v_fma(uy, uy, v_mul(uz, uz)));
-          const bool own_row = ybl + warp * RP + r < yrows;
-          const bool w0 = own_row && gx >= xb && gx < nx && !f.sol0;
-          const bool w1 = VX == 2 && own_row && gx >= xb && gx + 1 < nx && !f.sol1;
-          const long long zc = (long long)z * plane + in[r].t.o0;
           LBF_CHECK(a.flags, !(w0 || w1) || (z >= 0 && z < a.nz && in[r].t.o0 >= 0 && in[r].t.o0 < plane && zc + 9 * N < 10 * N));
           S* d0 = dst + zc;
           const T um = T(a.umax2);
@@ -1058,6 +1178,7 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
               red[1] += (w0 ? ux.x : 0.0f) + (w1 ? ux.y : 0.0f);
               red[2] += (w0 ? uy.x : 0.0f) + (w1 ? uy.y : 0.0f);
               red[3] += (w0 ? uz.x : 0.0f) + (w1 ? uz.y : 0.0f);
+              if constexpr (TWO != 0) red[4] += (w0 ? f.np[0].x : 0.0f) + (w1 ? f.np[0].y : 0.0f);
               red[5] += (w0 ? uu.x : 0.0f) + (w1 ? uu.y : 0.0f);
             }
           } else if (w0) {
@@ -1076,9 +1197,11 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
             red[1] += ux;
             red[2] += uy;
             red[3] += uz;
+            if constexpr (TWO != 0) red[4] += f.np[0];
             red[5] += uu;
           }
         }
+        fetch_new(in[r], f, it);
         // this plane becomes the one in flight: c_z = +1 of the plane below plus its own c_z = 0 part
         auto mid = [&](V u, V v) { return Q19 ? v_add(u, v) : v_fma(v, v_set<V>(T(4)), u); };
         {
