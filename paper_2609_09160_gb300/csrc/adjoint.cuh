@@ -77,6 +77,7 @@ __global__ void __launch_bounds__(FwdTile<BY>::THREADS)
   T* __restrict__ lout = static_cast<T*>(a.lam_out);
   const T* __restrict__ ffield = static_cast<const T*>(a.force_field);
 
+  grid_wait();
   const int lane = threadIdx.x, row = threadIdx.y;
   const int gx = blockIdx.x * FwdTile<BY>::XOUT - 1 + lane;
   const int gy = blockIdx.y * BY - 1 + row;

@@ -336,6 +336,29 @@ const void* mapped_host_pointer(const void* p) {
   return attr.type == cudaMemoryTypeHost ? attr.devicePointer : nullptr;
 }
 
+// A launch whose start may overlap the end of the kernel before it in the stream (programmatic dependent
+// launch); the kernel calls grid_wait() before it touches memory. It hides the launch and start-up of the
+// step's kernels (us a step, before -> after: 64 x 48 x 40 channel 10.3 -> 7.3, 524288 sites with a force
+// field 18.0 -> 15.7, droplet 128^3 113 -> 107). From about 2^23 sites on, grids of many waves gain nothing
+// and their first wave settles less evenly (512^3 FP16 1409 -> 1426), so those are launched as usual.
+cudaError_t launch_overlapped(const void* fn, dim3 grid, dim3 block, void** args, size_t smem, cudaStream_t st,
+                              long long sites) {
+  if (sites >= (1LL << 23)) return cudaLaunchKernel(fn, grid, block, args, smem, st);
+  cudaLaunchConfig_t cfg;
+  std::memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at;
+  std::memset(&at, 0, sizeof(at));
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelExC(&cfg, fn, args);
+}
+
 unsigned blocks_for(long long n, int threads) {
   long long b = (n + threads - 1) / threads;
   return (unsigned)std::max<long long>(1, std::min<long long>(b, 65535LL * 16));
@@ -422,9 +445,11 @@ dim3 phase_grid(const lbf_ctx* c) {
 
 template <class T>
 void launch_forces_T(lbf_ctx* c, int which) {
-  k_phase_forces<T><<<phase_grid(c), phase_block(), 0, c->stream>>>(
-      static_cast<const T*>(c->phi[which]), static_cast<T*>(c->F[which]), static_cast<T*>(c->G),
-      c->contrast ? static_cast<T*>(c->gphi) : nullptr, phase_params(c));
+  const T* phi = static_cast<const T*>(c->phi[which]);
+  T *F = static_cast<T*>(c->F[which]), *G = static_cast<T*>(c->G), *gphi = c->contrast ? static_cast<T*>(c->gphi) : nullptr;
+  PhaseParams pp = phase_params(c);
+  void* args[] = {&phi, &F, &G, &gphi, &pp};
+  launch_overlapped(reinterpret_cast<const void*>(&k_phase_forces<T>), phase_grid(c), phase_block(), args, 0, c->stream, c->N);
 }
 
 void launch_forces(lbf_ctx* c, int which) {
@@ -434,9 +459,12 @@ void launch_forces(lbf_ctx* c, int which) {
 
 template <class S, class T>
 void launch_advance_T(lbf_ctx* c) {
-  k_phase_advance<S, T><<<phase_grid(c), phase_block(), 0, c->stream>>>(
-      static_cast<const S*>(c->state[c->cur]), static_cast<const T*>(c->phi[c->pcur]), static_cast<const T*>(c->G),
-      static_cast<T*>(c->phi[1 - c->pcur]), phase_params(c));
+  const S* st = static_cast<const S*>(c->state[c->cur]);
+  const T *phi = static_cast<const T*>(c->phi[c->pcur]), *G = static_cast<const T*>(c->G);
+  T* phi_new = static_cast<T*>(c->phi[1 - c->pcur]);
+  PhaseParams pp = phase_params(c);
+  void* args[] = {&st, &phi, &G, &phi_new, &pp};
+  launch_overlapped(reinterpret_cast<const void*>(&k_phase_advance<S, T>), phase_grid(c), phase_block(), args, 0, c->stream, c->N);
 }
 
 void launch_advance(lbf_ctx* c) {
@@ -858,7 +886,7 @@ lbf_status launch_sep(lbf_ctx* c, const FwdParams& a, const void* src, void* dst
   void* args[] = {&as, &tr, &tt, &to};
   const dim3 block(32, k->threads / 32, 1);
   if (!c->sep_split) {
-    LBF_CUDA(cudaLaunchKernel(k->fn, c->sep.grid, block, args, k->smem, c->stream));
+    LBF_CUDA(launch_overlapped(k->fn, c->sep.grid, block, args, k->smem, c->stream, c->N));
     *done = true;
     return LBF_OK;
   }
@@ -948,7 +976,10 @@ lbf_status launch_forward(lbf_ctx* c, const void* src, void* dst, bool reduce) {
   }
   void* args[] = {&a, &tm, &sm};
   const dim3 grid(grid_x(c->nx, k->xout), grid_y(c->ny, k->by), c->fgrid.z);
-  LBF_CUDA(cudaLaunchKernel(k->fn, grid, dim3(32, k->threads / 32, 1), args, k->smem, c->stream));
+  if (k->store_map)  // the line-aligned kernel does not wait for its predecessor itself
+    LBF_CUDA(cudaLaunchKernel(k->fn, grid, dim3(32, k->threads / 32, 1), args, k->smem, c->stream));
+  else
+    LBF_CUDA(launch_overlapped(k->fn, grid, dim3(32, k->threads / 32, 1), args, k->smem, c->stream, c->N));
   return LBF_OK;
 }
 
@@ -1560,7 +1591,7 @@ lbf_status lbf_adjoint_step(lbf_ctx* c, const void* state_t, const void* state_t
   a.sc = c->sc;
   a.zchunk = c->zchunk;
   void* args[] = {&a};
-  LBF_CUDA(cudaLaunchKernel(c->adj.fn, c->agrid, dim3(32, c->adj.by + 2, 1), args, c->adj.smem, c->stream));
+  LBF_CUDA(launch_overlapped(c->adj.fn, c->agrid, dim3(32, c->adj.by + 2, 1), args, c->adj.smem, c->stream, c->N));
   return LBF_OK;
 }
 

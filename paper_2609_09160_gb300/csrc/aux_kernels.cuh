@@ -6,6 +6,7 @@
 #include <type_traits>
 
 #include "lattice.cuh"
+#include "tma.cuh"
 
 namespace lbf {
 
@@ -251,6 +252,7 @@ __global__ void __launch_bounds__(PhaseTile<T>::SITES, sizeof(T) == 4 ? 6 : 1) k
                                                                        const T* __restrict__ G,
                                                                        T* __restrict__ phi_new, PhaseParams p) {
   using PT = PhaseTile<T>;
+  grid_wait();
   __shared__ T sm[2][5][PT::SITES];  // phi, L_z phi, A_z V_x, A_z V_y, D_z V_z of the current plane
   const PhaseColumn c(p);
   const int me = threadIdx.y * 32 + threadIdx.x;
@@ -327,6 +329,7 @@ __global__ void __launch_bounds__(PhaseTile<T>::SITES, sizeof(T) == 4 ? 6 : 1) k
                                                                       T* __restrict__ F, T* __restrict__ G,
                                                                       T* __restrict__ gphi, PhaseParams p) {
   using PT = PhaseTile<T>;
+  grid_wait();
   __shared__ T sm[2][4][PT::SITES];  // A_z phi, D_z phi, phi, L_z phi of the current plane
   const PhaseColumn c(p);
   const int me = threadIdx.y * 32 + threadIdx.x;

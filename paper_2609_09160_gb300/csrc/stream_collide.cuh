@@ -581,6 +581,7 @@ __global__ void __launch_bounds__(FwdTile<BY>::THREADS, fwd_minb(L::Q, int(sizeo
   const S* __restrict__ src = static_cast<const S*>(a.src);
   S* __restrict__ dst = static_cast<S*>(a.dst);
   const T* __restrict__ ffield = static_cast<const T*>(a.force_field);
+  grid_wait();
 
   const int lane = threadIdx.x, row = threadIdx.y;
   const int x0 = blockIdx.x * FwdTile<BY>::XOUT;
@@ -1092,6 +1093,7 @@ __global__ void __launch_bounds__(FwdTile<BY>::THREADS, fwd_minb(L::Q, int(sizeo
     }
   }
 
+  grid_release();
   if (a.partials != nullptr) {
     // warp sums in the compute type, block and grid sums in FP64 (scratch: the idle ring)
     double* red_s = reinterpret_cast<double*>(smem_raw + RAW_BYTES);

@@ -825,6 +825,7 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
   };
 
   T red[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
+  grid_wait();  // nothing above touches what an earlier kernel writes
   if (warp == PAIRS) {
     // ---- the y halo rows: p of the one below the tile, m of the one above it ------------------------
     RowIn in[2] = {row_in(0), row_in(ROWS - 1)};
@@ -1260,6 +1261,7 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
     if (bad) atomicOr(a.flags, 1u);
   }
   __syncthreads();
+  grid_release();
 
   if (a.partials != nullptr) {
     // warp sums in the compute type, block and grid sums in FP64, in a fixed order

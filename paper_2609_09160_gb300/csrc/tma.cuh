@@ -92,6 +92,15 @@ __device__ __forceinline__ void bulk_wait_group0() { asm volatile("cp.async.bulk
 // orders this thread's generic-proxy shared-memory writes before later async-proxy (TMA) accesses
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
+// Programmatic dependent launch: a kernel launched with that attribute may start while its predecessor in
+// the stream still runs. grid_wait() returns when the predecessor is complete and its writes are visible
+// (at once without the attribute); grid_release() lets the successor's blocks start once every block has
+// called it or ended. It is called when a block's own work is done: called at its start, the successor's
+// blocks settle on whichever SMs have room first, and small grids then run two to an SM beside idle ones
+// (32^3 FP64 46.5 us a step against 33).
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
