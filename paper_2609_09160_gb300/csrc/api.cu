@@ -234,7 +234,7 @@ struct lbf_ctx {
   unsigned char* staging;
   Scales sc;
   cudaStream_t stream;
-  int zchunk, zchunk_phase;
+  int zchunk, zchunk_phase, azchunk;
   dim3 fgrid, agrid;
   KernelInfo fwd, adj;
   KernelInfo fwd_direct;  // the same step loading every site directly (sources TMA cannot read)
@@ -1217,7 +1217,19 @@ lbf_status lbf_create(lbf_ctx** out, const lbf_params* params, void* workspace, 
   // 512 x 1024 x 8 282.9 / 284.2 / 285.2, 96 x 90 x 70 59.0 / 63.7 / 68.7
   c->zchunk_phase = std::min(6, c->nz);
   c->fgrid = dim3(grid_x(c->nx, c->fwd.xout), grid_y(c->ny, c->fwd.by), (c->nz + c->zchunk - 1) / c->zchunk);
-  c->agrid = c->adj.fn ? dim3(grid_x(c->nx), grid_y(c->ny, c->adj.by), (c->nz + c->zchunk - 1) / c->zchunk) : dim3(1, 1, 1);
+  // the adjoint marches in chunks of its own: as short as whole waves of its CTAs allow on small lattices
+  // (128 x 64 x 64, us a launch at 4 / 5 / 6 / 7 / 8 planes: 34.5 / 35.7 / 26.2 / 29.7 / 32.4; 6 planes are
+  // 440 CTAs on 456 slots; the forward step's chunk, used before, was 8)
+  c->azchunk = c->zchunk;
+  c->agrid = dim3(1, 1, 1);
+  if (c->adj.fn != nullptr) {
+    int resident = 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, c->adj.fn, c->adj.threads, c->adj.smem) != cudaSuccess)
+      return cleanup(fail(LBF_ECUDA, std::string("device query failed: ") + cudaGetErrorString(cudaGetLastError())));
+    const long long ta = (long long)grid_x(c->nx) * grid_y(c->ny, c->adj.by);
+    c->azchunk = choose_zchunk_sep(c->nz, ta, double(sms) * std::max(resident, 1), 1.0);
+    c->agrid = dim3(grid_x(c->nx), grid_y(c->ny, c->adj.by), (c->nz + c->azchunk - 1) / c->azchunk);
+  }
   if (c->tma) {
     for (int k = 0; k < 2; ++k) {
       if ((st = encode_state_map(c, c->state[k], &c->tmap[k], c->fwd.box_x, c->fwd.by + 2)) != LBF_OK) return cleanup(st);
@@ -1589,7 +1601,7 @@ lbf_status lbf_adjoint_step(lbf_ctx* c, const void* state_t, const void* state_t
   a.nz = c->nz;
   a.N = c->N;
   a.sc = c->sc;
-  a.zchunk = c->zchunk;
+  a.zchunk = c->azchunk;
   void* args[] = {&a};
   LBF_CUDA(launch_overlapped(c->adj.fn, c->agrid, dim3(32, c->adj.by + 2, 1), args, c->adj.smem, c->stream, c->N));
   return LBF_OK;
