@@ -97,18 +97,37 @@ template <class V>
 struct PairSD {
   V S, D;
 };
-// p(x-1) + m(x+1) and p(x-1) - m(x+1) along x; h: the outer neighbour's value (edge lanes only)
-__device__ __forceinline__ PairSD<float2> x_sums(float2 p, float2 m, float h, int lane) {
-  float l = __shfl_up_sync(0xffffffffu, p.y, 1), r = __shfl_down_sync(0xffffffffu, m.x, 1);
-  if (lane == 0) l = h;
-  if (lane == 31) r = h;
+// p(x-1) + m(x+1) and p(x-1) - m(x+1) along x; the edge lanes take their outer neighbour h from the halo
+// (left, right), or, with AROUND, where a row is one tile long, by a shuffle that wraps around
+template <bool AROUND>
+struct Edge {
+  int lane;
+  bool left, right;
+  __device__ __forceinline__ float from_left(float v) const {
+    return AROUND ? __shfl_sync(0xffffffffu, v, (lane + 31) & 31) : __shfl_up_sync(0xffffffffu, v, 1);
+  }
+  __device__ __forceinline__ float from_right(float v) const {
+    return AROUND ? __shfl_sync(0xffffffffu, v, (lane + 1) & 31) : __shfl_down_sync(0xffffffffu, v, 1);
+  }
+  __device__ __forceinline__ double from_left(double v) const {
+    return AROUND ? __shfl_sync(0xffffffffu, v, (lane + 31) & 31) : __shfl_up_sync(0xffffffffu, v, 1);
+  }
+  __device__ __forceinline__ double from_right(double v) const {
+    return AROUND ? __shfl_sync(0xffffffffu, v, (lane + 1) & 31) : __shfl_down_sync(0xffffffffu, v, 1);
+  }
+};
+template <class E>
+__device__ __forceinline__ PairSD<float2> x_sums(float2 p, float2 m, float h, const E& e) {
+  float l = e.from_left(p.y), r = e.from_right(m.x);
+  if (e.left) l = h;
+  if (e.right) r = h;
   return {make_float2(l + m.y, p.x + r), make_float2(l - m.y, p.x - r)};
 }
-template <class T>
-__device__ __forceinline__ PairSD<T> x_sums(T p, T m, T h, int lane) {
-  T l = __shfl_up_sync(0xffffffffu, p, 1), r = __shfl_down_sync(0xffffffffu, m, 1);
-  if (lane == 0) l = h;
-  if (lane == 31) r = h;
+template <class E>
+__device__ __forceinline__ PairSD<double> x_sums(double p, double m, double h, const E& e) {
+  double l = e.from_left(p), r = e.from_right(m);
+  if (e.left) l = h;
+  if (e.right) r = h;
   return {l + r, l - r};
 }
 
@@ -378,6 +397,12 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
   const int z0 = blockIdx.z * a.zchunk;
   const int z1 = min(a.nz, z0 + a.zchunk);
   const int planes = z1 - z0 + 2;  // z0 - 1 .. z1, numbered 0 .. planes - 1
+  // rows of one tile (the tile's other edge is its x halo): the shuffles wrap around and nobody forms halo
+  // columns. Where lattices that small run: the short tile, and FP64 (32^3 FP64 33.1 -> 29.3 us a step); the
+  // indexed shuffles cost the large FP32 tile 2-3%
+  constexpr bool AROUND = SMALL || VX == 1;
+  const bool one_tile = AROUND && nx == XO;
+  const Edge<AROUND> edge = {lane, lane == 0 && !one_tile, lane == 31 && !one_tile};
   const bool dirty = MASK && a.tile_dirty[((long long)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] != 0;
 
   T keep = T(1) - pick<T>(a.omega, a.omega_f);
@@ -755,19 +780,19 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
       const V wp = v_add(c.by, c.eyz), wm = v_sub(c.by, c.eyz);
       const V tp = v_add(ap, c.exx), tm = v_add(am, c.exx), t0 = v_add(c.q0, c.exx);
       if constexpr (Q19) {
-        const PairSD<V> P = x_sums(v_add(tp, xp), v_sub(tp, xp), he[0], lane);
+        const PairSD<V> P = x_sums(v_add(tp, xp), v_sub(tp, xp), he[0], edge);
         put_y(0, ap, wp, c.eyy);
         own[0] = v_fma(ap, two, P.S);
         own[1] = P.D;
         own[2] = P.S;
-        const PairSD<V> M = x_sums(v_add(tm, xm), v_sub(tm, xm), he[1], lane);
+        const PairSD<V> M = x_sums(v_add(tm, xm), v_sub(tm, xm), he[1], edge);
         put_y(1, am, wm, c.eyy);
         own[3] = v_fma(am, two, M.S);
         own[4] = M.D;
         own[5] = M.S;
-        const PairSD<V> Z0 = x_sums(v_add(t0, c.bx), v_sub(t0, c.bx), he[2], lane);
-        const PairSD<V> Z1 = x_sums(v_add(c.by, c.exy), v_sub(c.by, c.exy), he[3], lane);
-        const PairSD<V> Z2 = x_sums(c.eyy, c.eyy, he[4], lane);
+        const PairSD<V> Z0 = x_sums(v_add(t0, c.bx), v_sub(t0, c.bx), he[2], edge);
+        const PairSD<V> Z1 = x_sums(v_add(c.by, c.exy), v_sub(c.by, c.exy), he[3], edge);
+        const PairSD<V> Z2 = x_sums(c.eyy, c.eyy, he[4], edge);
         const V X0 = v_fma(c.q0, two, Z0.S), X1 = v_fma(c.by, two, Z1.S), X2 = v_fma(c.eyy, two, Z2.S);
         put_y(2, X0, X1, X2);
         put_y(3, Z0.D, Z1.D, Z2.D);
@@ -776,11 +801,11 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
         own[7] = v_mul(Z0.D, two);
         own[8] = v_mul(Z0.S, two);
       } else {
-        const PairSD<V> Q2 = x_sums(c.eyy, c.eyy, he[6], lane);
+        const PairSD<V> Q2 = x_sums(c.eyy, c.eyy, he[6], edge);
         const V X2 = v_fma(c.eyy, four, Q2.S);
         auto part = [&](int k, V A, V B, V Y, V t) {  // constant, cx and cy coefficients, A + exx
-          const PairSD<V> Q0 = x_sums(v_add(t, B), v_sub(t, B), he[2 * k], lane);
-          const PairSD<V> Q1 = x_sums(v_add(Y, c.exy), v_sub(Y, c.exy), he[2 * k + 1], lane);
+          const PairSD<V> Q0 = x_sums(v_add(t, B), v_sub(t, B), he[2 * k], edge);
+          const PairSD<V> Q1 = x_sums(v_add(Y, c.exy), v_sub(Y, c.exy), he[2 * k + 1], edge);
           const V X0 = v_fma(A, four, Q0.S), X1 = v_fma(Y, four, Q1.S);
           put_y(3 * k, X0, X1, X2);
           put_y(3 * k + 1, Q0.D, Q1.D, Q2.D);
@@ -804,7 +829,7 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
           const V t = v_add(f[j], f[6 + j]);
-          q[j] = x_sums(v_add(t, f[3 + j]), v_sub(t, f[3 + j]), he[3 * k + j], lane);
+          q[j] = x_sums(v_add(t, f[3 + j]), v_sub(t, f[3 + j]), he[3 * k + j], edge);
           X[j] = v_fma(f[j], four, q[j].S);
         }
         put_y(3 * k, X[0], X[1], X[2]);
@@ -898,13 +923,15 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
     if constexpr (TMA) {
       for (int s = 0; s < STAGES - 1; ++s) issue(s);
     }
-    hfetch(0);
+    if (!one_tile) hfetch(0);
     int lost = -1;  // the plane whose wait gave up
     for (int it = -1; it < planes; ++it) {
       const int ip = it + 1;
       if (ip < planes) {
-        halo_columns(ht, hr < ROWS, ip, hraw0, hraw1, hext);
-        if (ip + 1 < planes) hfetch(ip + 1);
+        if (!one_tile) {
+          halo_columns(ht, hr < ROWS, ip, hraw0, hraw1, hext);
+          if (ip + 1 < planes) hfetch(ip + 1);
+        }
         if (TMA && !mbar_wait_bounded(&bars[ip % STAGES], uint32_t(ip / STAGES) & 1u, kWaitPolls)) {
           atomicOr(a.flags, 2u);
           lost = ip;
@@ -1053,14 +1080,18 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
         }
         if (it >= 2) {
           const int z = z0 + it - 2;
-          // the sums are in units of the smallest weight, 1/36 or 1/216. p* and u accumulate over the steps,
-          // so their factor is applied in two parts (vs rounded, and what it lacks): rounded once, it would
-          // scale them by 1 + 7e-9 (FP64 1 + 6e-17) in every step
+          // the sums are in units of the smallest weight, 1/36 or 1/216. In FP32 p* and u, which accumulate over
+          // the steps, take that factor in two parts (rounded, and what it lacks): rounded once, it would scale
+          // them by 1 + 7e-9 in every step (20 steps: error of u 9.1e-8 against 1.5e-7 with rounded weights)
           constexpr T sc = Q19 ? T(1) / T(36) : T(1) / T(216);
-          constexpr T lack = std::is_same<T, double>::value ? T(Q19 ? 1.5419764230904951e-18 : 2.569960705150825e-19)
-                                                            : T((Q19 ? 1.0 / 36.0 : 1.0 / 216.0) - double(sc));
+          constexpr T lack = T((Q19 ? 1.0 / 36.0 : 1.0 / 216.0) - double(sc));
           const V vs = v_set<V>(sc), vl = v_set<V>(lack);
-          auto scaled = [&](V v) -> V { return v_fma(v, vs, v_mul(v, vl)); };
+          auto scaled = [&](V v) -> V {
+            if constexpr (std::is_same<T, double>::value)
+              return v_mul(v, vs);
+            else
+              return v_fma(v, vs, v_mul(v, vl));
+          };
           const V b0 = scaled(f.a0);
           const bool own_row = ybl + warp * RP + r < yrows;
           const bool w0 = own_row && gx >= xb && gx < nx && !f.sol0;
