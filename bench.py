@@ -58,7 +58,7 @@ def measured_peaks():
 
 def kernel_source_sha():
     h = hashlib.sha1()
-    for name in ("lattice.cuh", "stream_collide.cuh", "stream_collide_aligned.cuh", "tma.cuh"):
+    for name in ("lattice.cuh", "stream_collide.cuh", "stream_collide_aligned.cuh", "stream_collide_sep.cuh", "tma.cuh"):
         with open(os.path.join(ROOT, "paper_2609_09160_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:12]
@@ -554,10 +554,11 @@ def kernel_label(s, lattice, storage, kind):
     lat = LATTICE_NAME[lattice]
     walls = kind in ("channel", "layered")
     if s.kernels_per_step == 2 and kind == "channel":
-        return (f"k_stream_collide_al<{lat},{storage},periodic> on the rows clear of the walls + "
+        return (f"k_stream_collide_sep<{lat},{storage},periodic> on the rows clear of the walls + "
                 f"k_stream_collide<{lat},{storage},mask> on the rows near them")
-    fused = (f"k_stream_collide<{lat},{storage},{'mask' if walls else 'periodic'}>" if walls or kind == "droplet"
-             else f"k_stream_collide_al or k_stream_collide<{lat},{storage},periodic> (the library's choice)")
+    if storage in ("f16", "bf16") and kind == "tg256":
+        return f"k_stream_collide or k_stream_collide_al<{lat},{storage},periodic> (the library's choice)"
+    fused = f"k_stream_collide_sep<{lat},{storage},{'mask' if walls else 'periodic'}>"
     if kind in ("droplet", "layered"):
         return f"k_phase_advance + k_phase_forces + {fused}"
     return fused

@@ -634,23 +634,7 @@ __global__ void __launch_bounds__(AlTile<S, TY>::THREADS, al_minb<L, S, TY, MASK
     if (last) {
       __threadfence();
       constexpr int NT = G::THREADS;
-      double* tree = reinterpret_cast<double*>(sbase);
-      for (int i = tid; i < 6 * 512; i += NT) tree[i] = 0.0;
-      __syncthreads();
-      for (int k = 0; k < 6; ++k) {
-        double acc = 0.0;
-        for (long long b = tid; b < nall; b += NT) acc += __ldcg(a.partials + b * 8 + k);
-        tree[k * 512 + tid] = acc;
-      }
-      __syncthreads();
-      for (int h = 256; h > 0; h >>= 1) {
-        for (int i = tid; i < 6 * h; i += NT) {
-          const int k = i / h, j = i % h;
-          tree[k * 512 + j] += tree[k * 512 + j + h];
-        }
-        __syncthreads();
-      }
-      if (tid < 6) a.sums[tid] = tree[tid * 512];
+      sum_partials<NT>(a.partials, nall, reinterpret_cast<double*>(sbase), a.sums, tid);
       if (tid == 0) *a.counter = 0u;
     }
   }

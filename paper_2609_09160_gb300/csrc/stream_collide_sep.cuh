@@ -169,7 +169,7 @@ constexpr size_t sep_smem_bytes() {
   using G = SepTile<L, S, VX, TY, RP>;
   const size_t need = 128 + STAGES * G::STAGEB + G::HXB + G::YB +
                       (MASK && !sep_cor_in_stage<S>() ? size_t(TY) * 10 * G::XO * sizeof(typename G::T) : 0);
-  return need < 6 * 512 * sizeof(double) + 256 ? 6 * 512 * sizeof(double) + 256 : need;
+  return need;
 }
 
 // Tile of a kernel: TY output rows, RP of them per warp, and the CTAs per SM asked of the register
@@ -1322,24 +1322,7 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
     if (last) {
       __threadfence();
       constexpr int NT = G::THREADS;
-      static_assert(NT <= 512, "final tree assumes <= 512 threads");
-      double* tree = reinterpret_cast<double*>(sbase);
-      for (int i = tid; i < 6 * 512; i += NT) tree[i] = 0.0;
-      __syncthreads();
-      for (int k = 0; k < 6; ++k) {
-        double acc = 0.0;
-        for (long long b = tid; b < nall; b += NT) acc += __ldcg(a.partials + b * 8 + k);
-        tree[k * 512 + tid] = acc;
-      }
-      __syncthreads();
-      for (int h = 256; h > 0; h >>= 1) {
-        for (int i = tid; i < 6 * h; i += NT) {
-          const int k = i / h, j = i % h;
-          tree[k * 512 + j] += tree[k * 512 + j + h];
-        }
-        __syncthreads();
-      }
-      if (tid < 6) a.sums[tid] = tree[tid * 512];
+      sum_partials<NT>(a.partials, nall, reinterpret_cast<double*>(sbase), a.sums, tid);
       if (tid == 0) *a.counter = 0u;
     }
   }
