@@ -35,11 +35,12 @@
 //
 // What bounds it (one GB300; GLUPS, same workloads, before -> after; "before" is the faster of the two
 // population-ring kernels):
-//   D3Q19 FP32 512^3 64.6 -> 71, 256^3 57.0 -> 68; FP16 512^3 65.5 -> 95; D3Q27 FP32 512^3 51.8 -> 64.3,
-//   FP16 53.6 -> 71.5; D3Q27h FP32 256^3 31.6 -> 39.4, FP16 29.8 -> 38.7; D3Q19 FP64 32^3 0.43 -> 0.94.
-//   225 thread instructions per site on D3Q19 FP32 against 423. FP32 moves DRAM at 5.7 TB/s of 6.7 (reads
-//   1.04x the state); 16-bit storage and D3Q27 are bound by the latency of the two halves of a plane's work
-//   with 12 to 16 warps per SM (shared-memory pipe 50-57% busy, issue 38-55%).
+//   D3Q19 FP32 512^3 64.6 -> 70, 256^3 57.0 -> 67; FP16 512^3 65.5 -> 94; D3Q27 FP32 512^3 51.8 -> 64,
+//   FP16 53.6 -> 71.5; D3Q27h FP32 256^3 31.6 -> 39.4, FP16 29.8 -> 38.7; D3Q19 FP64 32^3 0.43 -> 1.13.
+//   Thread instructions per site: D3Q19 FP32 188 (421 before), FP16 245, D3Q27 FP32 305 (600), D3Q27h 460
+//   (970). FP32 moves DRAM at 5.6 TB/s of 6.7 (reads 1.03x the state); 16-bit storage and the D3Q27 lattices
+//   are bound by the latency of the two halves of a plane's work with 8 to 16 warps per SM (shared-memory
+//   pipe 40-66% busy, issue 45-55%; top stalls barrier and fixed latency).
 // Why this split:
 //   * two rows per warp (RP = 2): a row pair exchanges p and m in registers, which halves the shared-memory
 //     exchange; D3Q19 FP16 84 -> 92 with 12 warps of 168 registers instead of 16 of 110. The D3Q27 lattices
