@@ -647,8 +647,13 @@ int choose_zchunk(int nz, long long tiles, double resident) {
   return std::min(zc, nz);
 }
 
+// planes per CTA of the masked launch of a split step: beside the line-aligned kernel, and beside the
+// axis-separated one, whose CTAs take most of the shared memory
 #ifndef LBF_SPLIT_ZCHUNK
-#define LBF_SPLIT_ZCHUNK 8
+#define LBF_SPLIT_ZCHUNK 32
+#endif
+#ifndef LBF_SEP_SPLIT_ZCHUNK
+#define LBF_SEP_SPLIT_ZCHUNK 8
 #endif
 
 // the side stream of a split step
@@ -767,12 +772,13 @@ lbf_status setup_sep(lbf_ctx* c, const lbf_params* p, const Layout& L, int sms, 
   const bool forced = kname == "sep" || kname == "sepsmall";
   if (!sep_built(p) || !(kname.empty() || forced)) return LBF_OK;
   if (storage_bytes(c->storage) == 2 && c->nx % 2 != 0) return LBF_OK;  // no 4-byte aligned pairs of sites
-  // 16-bit storage without walls: a stored value is rounded by the last bits of its FP32 result, so another
-  // order of summation draws other, equally good roundings. Where nothing drives the flow the sums of p* and u
-  // cancel, and on small lattices what is left is that noise (sums of 5.3M BF16 sites after 51 steps: 1.4e-4
-  // apart, both 5e-4 from FP64; it falls as 1 / sites). Those lattices keep the 30-column kernel and its values
-  if (storage_bytes(c->storage) == 2 && !c->has_mask && !forced && c->N < (c->storage == LBF_F16 ? 1LL << 25 : 1LL << 26))
-    return LBF_OK;
+  // 16-bit storage keeps the kernels whose roundings it has, with and without walls. A stored p* or u is the
+  // FP32 result rounded to 2^-11 (FP16) or 2^-8 (BF16) of itself, up or down as its last bits decide, so another
+  // order of summation draws other, equally good roundings: each moves the sum of a conserved moment by up to one
+  // unit, and after n steps two such runs of N sites of size u differ by about unit * u * sqrt(n N) in sums that
+  // grow only with what drives the flow (that cancel where nothing does). No lattice size brings that below FP32
+  // rounding for every n, so the axis-separated kernel is taken here only on request (LBF_KERNEL=sep, sepsmall)
+  if (storage_bytes(c->storage) == 2 && !forced) return LBF_OK;
   const bool field = p->force_field != nullptr;
   // below about 2^20 sites the tall tiles leave SMs idle: short ones (ensemble members, 524288 sites with
   // walls and a force field: 17 us a step against 20.6)
@@ -800,7 +806,7 @@ lbf_status setup_sep(lbf_ctx* c, const lbf_params* p, const Layout& L, int sms, 
     c->sep.y_rows = len;
     c->dirty_begin = (begin + len) % c->ny;
     c->dirty_rows = c->ny - len;
-    c->zchunk_dirty = std::min(LBF_SPLIT_ZCHUNK, c->nz);
+    c->zchunk_dirty = std::min(LBF_SEP_SPLIT_ZCHUNK, c->nz);
     c->grid_dirty = dim3(grid_x(c->nx, c->fwd.xout), grid_y(c->dirty_rows, c->fwd.by), (c->nz + c->zchunk_dirty - 1) / c->zchunk_dirty);
   }
   c->sep.async = kernel(false);
