@@ -247,12 +247,10 @@ struct PhaseColumn {
 // With walls, u is taken as 0 at solid sites and phi is not advanced there (it keeps its value),
 // so a wall in contact with one bulk phase exchanges no phi.
 template <class S, class T>
-__global__ void __launch_bounds__(PhaseTile<T>::SITES, sizeof(T) == 4 ? 6 : 1) k_phase_advance(const S* __restrict__ st,
-                                                                       const T* __restrict__ phi,
-                                                                       const T* __restrict__ G,
-                                                                       T* __restrict__ phi_new, PhaseParams p) {
+__global__ void __launch_bounds__(PhaseTile<T>::SITES, sizeof(T) == 4 ? 6 : 1)
+    k_phase_advance(const S* st, const T* phi, const T* G, T* phi_new, PhaseParams p) {
   using PT = PhaseTile<T>;
-  grid_wait();
+  grid_wait();  // then plain, coherent loads (no __restrict__): the predecessor may still have been writing
   __shared__ T sm[2][5][PT::SITES];  // phi, L_z phi, A_z V_x, A_z V_y, D_z V_z of the current plane
   const PhaseColumn c(p);
   const int me = threadIdx.y * 32 + threadIdx.x;
@@ -325,11 +323,10 @@ __global__ void __launch_bounds__(PhaseTile<T>::SITES, sizeof(T) == 4 ? 6 : 1) k
 // With a density contrast grad phi is also written (gphi, else null): the fused step forms the
 // pressure and viscous-gradient forces from it and the raw moments of the new state.
 template <class T>
-__global__ void __launch_bounds__(PhaseTile<T>::SITES, sizeof(T) == 4 ? 6 : 1) k_phase_forces(const T* __restrict__ phi,
-                                                                      T* __restrict__ F, T* __restrict__ G,
-                                                                      T* __restrict__ gphi, PhaseParams p) {
+__global__ void __launch_bounds__(PhaseTile<T>::SITES, sizeof(T) == 4 ? 6 : 1)
+    k_phase_forces(const T* phi, T* F, T* G, T* gphi, PhaseParams p) {
   using PT = PhaseTile<T>;
-  grid_wait();
+  grid_wait();  // then plain, coherent loads, as above
   __shared__ T sm[2][4][PT::SITES];  // A_z phi, D_z phi, phi, L_z phi of the current plane
   const PhaseColumn c(p);
   const int me = threadIdx.y * 32 + threadIdx.x;

@@ -103,21 +103,21 @@ struct Codec;
 template <>
 struct Codec<double> {
   static constexpr bool scaled = false;
-  __device__ __forceinline__ static double load(const double* p) { return __ldg(p); }
+  __device__ __forceinline__ static double load(const double* p) { return *p; }
   __device__ __forceinline__ static void store(double* p, double v) { *p = v; }
   __device__ __forceinline__ static void store_sr(double* p, double v, uint32_t) { *p = v; }
 };
 template <>
 struct Codec<float> {
   static constexpr bool scaled = false;
-  __device__ __forceinline__ static float load(const float* p) { return __ldg(p); }
+  __device__ __forceinline__ static float load(const float* p) { return *p; }
   __device__ __forceinline__ static void store(float* p, float v) { *p = v; }
   __device__ __forceinline__ static void store_sr(float* p, float v, uint32_t) { *p = v; }
 };
 template <>
 struct Codec<__half> {
   static constexpr bool scaled = true;
-  __device__ __forceinline__ static float load(const __half* p) { return __half2float(__ldg(p)); }
+  __device__ __forceinline__ static float load(const __half* p) { return __half2float(*p); }
   __device__ __forceinline__ static void store(__half* p, float v) { *p = __float2half_rn(v); }
   // FP16 keeps 10 of FP32's 23 significand bits: 13 random bits, then round toward zero
   __device__ __forceinline__ static void store_sr(__half* p, float v, uint32_t r) {
@@ -128,7 +128,7 @@ template <>
 struct Codec<__nv_bfloat16> {
   static constexpr bool scaled = true;
   __device__ __forceinline__ static float load(const __nv_bfloat16* p) {
-    return __bfloat162float(__ldg(p));
+    return __bfloat162float(*p);
   }
   __device__ __forceinline__ static void store(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
   // BF16 is the upper half of FP32: 16 random bits, then truncation

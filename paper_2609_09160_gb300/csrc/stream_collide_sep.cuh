@@ -384,9 +384,11 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
   __shared__ __align__(8) uint64_t bars[STAGES];
   __shared__ volatile int gave_up[2];
 
-  const S* __restrict__ src = static_cast<const S*>(a.src);
-  S* __restrict__ dst = static_cast<S*>(a.dst);
-  const T* __restrict__ ffield = static_cast<const T*>(a.force_field);
+  // an overlapped launch is alive while its predecessor writes: everything but the wall tables is read by plain,
+  // coherent loads (no __restrict__, no __ldg), which stay behind grid_wait()
+  const S* src = static_cast<const S*>(a.src);
+  S* dst = static_cast<S*>(a.dst);
+  const T* ffield = static_cast<const T*>(a.force_field);
 
   const int lane = threadIdx.x, warp = __shfl_sync(0xffffffffu, int(threadIdx.y), 0);  // warp-uniform
   const int nx = a.nx, ny = a.ny;
@@ -447,8 +449,8 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
     const S* b = src + (long long)wrap(z0 - 1 + ip, a.nz) * plane;
 #pragma unroll
     for (int k = 0; k < 10; ++k) {
-      v0[k] = __ldg(b + k * N + t.o0);
-      if constexpr (VX == 2) v1[k] = __ldg(b + k * N + t.o1);
+      v0[k] = b[k * N + t.o0];
+      if constexpr (VX == 2) v1[k] = b[k * N + t.o1];
     }
   };
   auto fetch_extra = [&](const Site& t, int ip, Extra& r) {
@@ -457,8 +459,8 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
     if constexpr (FF) {
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
-        r.f0[k] = __ldg(ffield + k * N + zoff + t.o0);
-        if constexpr (VX == 2) r.f1[k] = __ldg(ffield + k * N + zoff + t.o1);
+        r.f0[k] = ffield[k * N + zoff + t.o0];
+        if constexpr (VX == 2) r.f1[k] = ffield[k * N + zoff + t.o1];
       }
     }
     if constexpr (TWO != 0) {
@@ -468,19 +470,19 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
       if (TMA && VX == 2 && t.o1 == t.o0 + 1) {
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-          const float2 q = __ldg(reinterpret_cast<const float2*>(Fo + k * N + t.o0));
+          const float2 q = *reinterpret_cast<const float2*>(Fo + k * N + t.o0);
           r.f0[k] = q.x, r.f1[k] = q.y;
         }
-        const float2 q = __ldg(reinterpret_cast<const float2*>(po + t.o0));
+        const float2 q = *reinterpret_cast<const float2*>(po + t.o0);
         r.p0 = q.x, r.p1 = q.y;
       } else {
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-          r.f0[k] = __ldg(Fo + k * N + t.o0);
-          if constexpr (VX == 2) r.f1[k] = __ldg(Fo + k * N + t.o1);
+          r.f0[k] = Fo[k * N + t.o0];
+          if constexpr (VX == 2) r.f1[k] = Fo[k * N + t.o1];
         }
-        r.p0 = __ldg(po + t.o0);
-        if constexpr (VX == 2) r.p1 = __ldg(po + t.o1);
+        r.p0 = po[t.o0];
+        if constexpr (VX == 2) r.p1 = po[t.o1];
       }
     }
     if constexpr (MASK) {

@@ -94,7 +94,9 @@ __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.p
 
 // Programmatic dependent launch: a kernel launched with that attribute may start while its predecessor in
 // the stream still runs. grid_wait() returns when the predecessor is complete and its writes are visible
-// (at once without the attribute); grid_release() lets the successor's blocks start once every block has
+// (at once without the attribute); what the predecessor may have written is read by plain loads after it, since
+// ld.global.nc (__ldg, const __restrict__) is for data that nobody writes while the kernel runs and may be moved
+// above the wait; grid_release() lets the successor's blocks start once every block has
 // called it or ended. It is called when a block's own work is done: called at its start, the successor's
 // blocks settle on whichever SMs have room first, and small grids then run two to an SM beside idle ones
 // (32^3 FP64 46.5 us a step against 33).
