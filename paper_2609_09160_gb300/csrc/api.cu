@@ -116,6 +116,10 @@ int fwd_by(int lattice, int storage, bool mask, bool two) {
                           lattice == LBF_D3Q27H);
 }
 int min_zchunk(int nz) { return std::min(8, nz); }
+// gridDim.y and gridDim.z end at 65535: the fewest planes per CTA that keep a grid of z-chunks within it
+constexpr int kGridMax = 65535;
+int grid_min_z(int nz) { return (nz - 1) / kGridMax + 1; }
+bool grid_fits(const dim3& g) { return g.y <= unsigned(kGridMax) && g.z <= unsigned(kGridMax); }
 // output rows of the line-aligned kernel for these parameters (0 when it is not built for them)
 int aligned_by(const lbf_params* p) {
   if (p->two_component || p->populations || p->storage == LBF_F64) return 0;
@@ -787,7 +791,7 @@ lbf_status setup_sep(lbf_ctx* c, const lbf_params* p, const Layout& L, int sms, 
   // large lattices whose rows TMA cannot take: the 30-column kernel (333 x 250 x 189, GLUPS: 38.0 against
   // 34.8 with the best tile of this one)
   if (!rows_tma && !small && !forced && !c->two) return LBF_OK;
-  bool walls = c->has_mask;
+  bool walls = c->has_mask, split = false;
   c->sep.y_begin = 0;
   c->sep.y_rows = c->ny;
   const int two = c->two ? (c->contrast ? 2 : 1) : 0;
@@ -801,12 +805,12 @@ lbf_status setup_sep(lbf_ctx* c, const lbf_params* p, const Layout& L, int sms, 
     if (!clean_band(c, p, k.by, &begin, &len)) return LBF_OK;  // scattered walls: the 30-column
     // kernel (192 x 160 x 176, 20% solid, GLUPS: 33.7 against 33.3 with the short tile, 25.9 with the tall one)
     walls = false;
-    c->sep_split = true;
+    split = true;
     c->sep.y_begin = begin;
     c->sep.y_rows = len;
     c->dirty_begin = (begin + len) % c->ny;
     c->dirty_rows = c->ny - len;
-    c->zchunk_dirty = std::min(LBF_SEP_SPLIT_ZCHUNK, c->nz);
+    c->zchunk_dirty = std::max(std::min(LBF_SEP_SPLIT_ZCHUNK, c->nz), grid_min_z(c->nz));
     c->grid_dirty = dim3(grid_x(c->nx, c->fwd.xout), grid_y(c->dirty_rows, c->fwd.by), (c->nz + c->zchunk_dirty - 1) / c->zchunk_dirty);
   }
   c->sep.async = kernel(false);
@@ -820,21 +824,25 @@ lbf_status setup_sep(lbf_ctx* c, const lbf_params* p, const Layout& L, int sms, 
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, k.fn, k.threads, k.smem) != cudaSuccess)
     return fail(LBF_ECUDA, std::string("device query failed: ") + cudaGetErrorString(cudaGetLastError()));
   const long long tiles = (long long)grid_x(c->nx, k.xout) * grid_y(c->sep.y_rows, k.by);
-  c->sep.zchunk = choose_zchunk_sep(c->nz, tiles, double(sms) * std::max(resident, 1), c->sep_split ? 2.0 : 1.0);
+  c->sep.zchunk = choose_zchunk_sep(c->nz, tiles, double(sms) * std::max(resident, 1), split ? 2.0 : 1.0);
   if (const char* e = std::getenv("LBF_ZCHUNK")) {
     const int v = std::atoi(e);
     if (v >= 1) c->sep.zchunk = std::min(c->nz, std::max(sep_min_z(c->nz, tiles), v));
   }
   c->sep.grid = dim3(grid_x(c->nx, k.xout), grid_y(c->sep.y_rows, k.by), (c->nz + c->sep.zchunk - 1) / c->sep.zchunk);
+  // its tiles are lower than those of the 30-column kernel (FP64 2 rows against 4): lattices of more rows than
+  // its grid holds keep that one
+  if (!grid_fits(c->sep.grid) || (split && !grid_fits(c->grid_dirty))) return LBF_OK;
   const long long blocks = (long long)c->sep.grid.x * c->sep.grid.y * c->sep.grid.z +
-                           (c->sep_split ? (long long)c->grid_dirty.x * c->grid_dirty.y * c->grid_dirty.z : 0);
+                           (split ? (long long)c->grid_dirty.x * c->grid_dirty.y * c->grid_dirty.z : 0);
   if (blocks > L.npartials) return fail(LBF_EINTERNAL, "partials buffer too small");
   for (int i = 0; i < 2 && c->sep.tma.fn != nullptr; ++i)
     if ((st = encode_row_map(c, c->state[i], &c->sep.row[i], k.box_x, 1)) != LBF_OK ||
         (st = encode_row_map(c, c->state[i], &c->sep.tile[i], k.box_x, k.by + 2)) != LBF_OK ||
         (st = encode_row_map(c, c->state[i], &c->sep.out[i], k.box_x, k.out_rows)) != LBF_OK)
       return st;
-  if (c->sep_split && (st = create_side(c)) != LBF_OK) return st;
+  if (split && (st = create_side(c)) != LBF_OK) return st;
+  c->sep_split = split;
   c->sep.on = true;
   return LBF_OK;
 }
@@ -1229,7 +1237,7 @@ lbf_status lbf_create(lbf_ctx** out, const lbf_params* params, void* workspace, 
   // phase-field kernels: short chunks fill the chip on small lattices and cost the large ones nothing (the
   // restaged planes hit L2). us a step at 6 / 11 / 15 planes: droplet 128^3 113.0 / 113.7 / 114.5, layered
   // 512 x 1024 x 8 282.9 / 284.2 / 285.2, 96 x 90 x 70 59.0 / 63.7 / 68.7
-  c->zchunk_phase = std::min(6, c->nz);
+  c->zchunk_phase = std::max(std::min(6, c->nz), grid_min_z(c->nz));
   c->fgrid = dim3(grid_x(c->nx, c->fwd.xout), grid_y(c->ny, c->fwd.by), (c->nz + c->zchunk - 1) / c->zchunk);
   // the adjoint marches in chunks of its own: as short as whole waves of its CTAs allow on small lattices
   // (128 x 64 x 64, us a launch at 4 / 5 / 6 / 7 / 8 planes: 34.5 / 35.7 / 26.2 / 29.7 / 32.4; 6 planes are
@@ -1241,7 +1249,7 @@ lbf_status lbf_create(lbf_ctx** out, const lbf_params* params, void* workspace, 
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, c->adj.fn, c->adj.threads, c->adj.smem) != cudaSuccess)
       return cleanup(fail(LBF_ECUDA, std::string("device query failed: ") + cudaGetErrorString(cudaGetLastError())));
     const long long ta = (long long)grid_x(c->nx) * grid_y(c->ny, c->adj.by);
-    c->azchunk = choose_zchunk_sep(c->nz, ta, double(sms) * std::max(resident, 1), 1.0);
+    c->azchunk = std::max(choose_zchunk_sep(c->nz, ta, double(sms) * std::max(resident, 1), 1.0), grid_min_z(c->nz));
     c->agrid = dim3(grid_x(c->nx), grid_y(c->ny, c->adj.by), (c->nz + c->azchunk - 1) / c->azchunk);
   }
   if (c->tma) {
