@@ -133,13 +133,15 @@ bool sep_built(const lbf_params* p) {
   if (p->two_component) return p->lattice == LBF_D3Q19 && p->storage == LBF_F32;
   return !p->populations && !(p->lattice == LBF_D3Q27H && p->mask != nullptr);
 }
-// z-chunks of the axis-separated kernel: at most kSepMaxZ planes, at least two and no fewer than keep a grid
-// of `tiles` columns within kSepBlocks blocks (one 64-byte partial sum each) where that is possible
+// z-chunks of the axis-separated kernel: at most kSepMaxZ planes (64 with one FP32 row per warp, whose threads add
+// up their sums over a whole chunk), at least two and no fewer than keep a grid of `tiles` columns within
+// kSepBlocks blocks (one 64-byte partial sum each) where that is possible
 constexpr int kSepMaxZ = 96;
+int sep_max_z(int rp, int storage) { return rp > 1 || storage == LBF_F64 ? kSepMaxZ : 64; }
 constexpr long long kSepBlocks = 1 << 16;
-int sep_min_z(int nz, long long tiles) {
+int sep_min_z(int nz, long long tiles, int zmax) {
   int z = std::min(2, nz);
-  while (z < std::min(kSepMaxZ, nz) && tiles * ((nz + z - 1) / z) > kSepBlocks) ++z;
+  while (z < std::min(zmax, nz) && tiles * ((nz + z - 1) / z) > kSepBlocks) ++z;
   return z;
 }
 // tiles of its largest grid, over both tile heights (walls may add the masked kernel's rows)
@@ -150,7 +152,7 @@ long long sep_max_tiles(const lbf_params* p) {
                                   : std::min(sep_config(Q, bytes, high, false).ty, sep_config(Q, bytes, high, true).ty);
   const long long tiles = (long long)grid_x(p->nx, 32 * sep_vx(bytes)) * grid_y(p->ny, ty);
   // fewer columns (the taller tile, the rows of a split) may be cut into more chunks: up to kSepBlocks
-  const int zc = sep_min_z(p->nz, tiles);
+  const int zc = sep_min_z(p->nz, tiles, sep_max_z(1, p->storage));
   return std::max(tiles * ((p->nz + zc - 1) / zc), std::min(kSepBlocks, tiles * ((p->nz + 1) / 2)));
 }
 
@@ -598,14 +600,14 @@ lbf_status encode_row_map(const lbf_ctx* c, const void* base, CUtensorMap* out, 
 // planes: FP32 70.5 / 73.1 / 73.4 / 72.9 / 72.8, FP16 96.3 / 96.7 / 95.7 / 92.2 / 83.1). Beside the rows near
 // walls of a split step the chunks leave at least two waves (min_waves): those CTAs hold SMs as well
 // (200 x 163 x 187 BF16: 24-plane chunks 55.8, 47-plane chunks, one wave, 43.2).
-int choose_zchunk_sep(int nz, long long tiles, double resident, double min_waves) {
-  const int zmin = sep_min_z(nz, tiles);
-  int zc = std::min(nz, kSepMaxZ);
+int choose_zchunk_sep(int nz, long long tiles, double resident, double min_waves, int zmax) {
+  const int zmin = sep_min_z(nz, tiles, zmax);
+  int zc = std::min(nz, zmax);
   double best = 1e30;
   for (int chunks = 1; chunks <= nz; ++chunks) {
     const int z = (nz + chunks - 1) / chunks;
     if (z < zmin) break;
-    if (z > kSepMaxZ) continue;
+    if (z > zmax) continue;
     const long long nchunks = (nz + z - 1) / z;
     const double waves = double(tiles * nchunks) / resident;
     // many waves run into one another: the last one costs half of itself on average
@@ -824,10 +826,11 @@ lbf_status setup_sep(lbf_ctx* c, const lbf_params* p, const Layout& L, int sms, 
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, k.fn, k.threads, k.smem) != cudaSuccess)
     return fail(LBF_ECUDA, std::string("device query failed: ") + cudaGetErrorString(cudaGetLastError()));
   const long long tiles = (long long)grid_x(c->nx, k.xout) * grid_y(c->sep.y_rows, k.by);
-  c->sep.zchunk = choose_zchunk_sep(c->nz, tiles, double(sms) * std::max(resident, 1), split ? 2.0 : 1.0);
+  const int zmax = sep_max_z(k.out_rows, c->storage);
+  c->sep.zchunk = choose_zchunk_sep(c->nz, tiles, double(sms) * std::max(resident, 1), split ? 2.0 : 1.0, zmax);
   if (const char* e = std::getenv("LBF_ZCHUNK")) {
     const int v = std::atoi(e);
-    if (v >= 1) c->sep.zchunk = std::min(c->nz, std::max(sep_min_z(c->nz, tiles), v));
+    if (v >= 1) c->sep.zchunk = std::min({c->nz, zmax, std::max(sep_min_z(c->nz, tiles, zmax), v)});
   }
   c->sep.grid = dim3(grid_x(c->nx, k.xout), grid_y(c->sep.y_rows, k.by), (c->nz + c->sep.zchunk - 1) / c->sep.zchunk);
   // its tiles are lower than those of the 30-column kernel (FP64 2 rows against 4): lattices of more rows than
@@ -1249,7 +1252,7 @@ lbf_status lbf_create(lbf_ctx** out, const lbf_params* params, void* workspace, 
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, c->adj.fn, c->adj.threads, c->adj.smem) != cudaSuccess)
       return cleanup(fail(LBF_ECUDA, std::string("device query failed: ") + cudaGetErrorString(cudaGetLastError())));
     const long long ta = (long long)grid_x(c->nx) * grid_y(c->ny, c->adj.by);
-    c->azchunk = std::max(choose_zchunk_sep(c->nz, ta, double(sms) * std::max(resident, 1), 1.0), grid_min_z(c->nz));
+    c->azchunk = std::max(choose_zchunk_sep(c->nz, ta, double(sms) * std::max(resident, 1), 1.0, kSepMaxZ), grid_min_z(c->nz));
     c->agrid = dim3(grid_x(c->nx), grid_y(c->ny, c->adj.by), (c->nz + c->azchunk - 1) / c->azchunk);
   }
   if (c->tma) {

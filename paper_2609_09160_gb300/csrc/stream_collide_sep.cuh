@@ -383,6 +383,11 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
   T* corb = yv + G::YB / sizeof(T);                                    // [TY][10][XO] (MASK, where needed)
   __shared__ __align__(8) uint64_t bars[STAGES];
   __shared__ volatile int gave_up[2];
+  // with two rows a thread adds up to 192 pairs in a chunk: in FP32 its sums go to FP64 every 32 planes, after at
+  // most 64 additions (a uniform flow's sums over 96 planes: 8e-7 off instead of 2.3e-6). With one row the chunks
+  // are of at most 64 planes
+  constexpr bool PARTS = RP == 2 && std::is_same<T, float>::value;
+  __shared__ double parts[PARTS ? G::WARPS * 6 : 1];  // a warp's sums so far
 
   // an overlapped launch is alive while its predecessor writes: everything but the wall tables is read by plain,
   // coherent loads (no __restrict__, no __ldg), which stay behind grid_wait()
@@ -853,6 +858,13 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
   };
 
   T red[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
+  if (PARTS && lane < 6) parts[warp * 6 + lane] = 0.0;
+  __syncwarp();
+  auto warp_sum = [](T v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return static_cast<double>(v);
+  };
   grid_wait();  // nothing above touches what an earlier kernel writes
   if (warp == PAIRS) {
     // ---- the y halo rows: p of the one below the tile, m of the one above it ------------------------
@@ -1010,284 +1022,298 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
     }
     const bool by_tma = TMA && !dirty && x0 == xb && ybl + warp * RP + RP <= yrows && gy[RP - 1] == gy[0] + RP - 1;
     cta_barrier<G::THREADS>();
-    for (int it = 0; it < planes && !gave_up[(it - 1) & 1]; ++it) {
-      V F[RP][3], own[RP][9];
-      V pin[RP > 1 ? NY : 1], min_[RP > 1 ? NY : 1];  // p of the lower, m of the upper of two rows
-      bool s0[RP], s1[RP];
-      copies_done();
-#pragma unroll
-      for (int r = 0; r < RP; ++r) {
-        V P[NY], M[NY];
-        row_front(in[r], it, true, F[r], P, M, own[r]);
-        if (r == 0 && warp > 0) {
-#pragma unroll
-          for (int e = 0; e < NY; ++e) *y_at(it, 1, e, warp - 1) = M[e];
-        }
-        if (r == RP - 1 && warp < PAIRS - 1) {
-#pragma unroll
-          for (int e = 0; e < NY; ++e) *y_at(it, 0, e, warp + 1) = P[e];
-        }
-        if constexpr (RP > 1) {
-#pragma unroll
-          for (int e = 0; e < NY; ++e) {
-            if (r == 0) pin[e] = P[e];
-            else min_[e] = M[e];
+    int it = 0;
+    do {
+      const int part = PARTS ? min(planes, it + 32) : planes;
+      for (; it < part && !gave_up[(it - 1) & 1]; ++it) {
+        V F[RP][3], own[RP][9];
+        V pin[RP > 1 ? NY : 1], min_[RP > 1 ? NY : 1];  // p of the lower, m of the upper of two rows
+        bool s0[RP], s1[RP];
+        copies_done();
+  #pragma unroll
+        for (int r = 0; r < RP; ++r) {
+          V P[NY], M[NY];
+          row_front(in[r], it, true, F[r], P, M, own[r]);
+          if (r == 0 && warp > 0) {
+  #pragma unroll
+            for (int e = 0; e < NY; ++e) *y_at(it, 1, e, warp - 1) = M[e];
           }
-        }
-        s0[r] = MASK && (in[r].e.l0 >> 31) != 0u;
-        s1[r] = MASK && (in[r].e.l1 >> 31) != 0u;
-        if constexpr (AHEAD) {
-          if (it + 1 < planes) fetch(in[r], it + 1);
-        }
-        // c_z = -1 part of the plane below, as far as it needs no neighbour row
-        Flight& f = fl[r];
-        f.rzz = v_add(MASK ? f.rzz : f.jz, own[r][3]);
-        f.a0 = v_add(f.a0, own[r][3]);
-        f.jz = v_sub(f.jz, own[r][3]);
-        f.jx = v_add(f.jx, own[r][4]);
-        f.rxz = v_sub(f.rxz, own[r][4]);
-        f.rxx = v_add(f.rxx, own[r][5]);
-      }
-      if constexpr (TMA) {
-        bulk_wait_group_read0();  // the last outputs have left their stage
-      } else {
-#pragma unroll
-        for (int r = 0; r < RP; ++r) copy_row(in[r], it - 1 + STAGES);  // into the stage of plane it - 1
-        copies_group();
-      }
-      cta_barrier<G::THREADS>();
-#pragma unroll
-      for (int r = 0; r < RP; ++r) {
-        Flight& f = fl[r];
-        const int row = in[r].t.row;
-        auto y_sums = [&](int e) -> PairSD<V> {
-          const V l = r == 0 ? *y_at(it, 0, e, warp) : pin[RP > 1 ? e : 0];
-          const V h = r == RP - 1 ? *y_at(it, 1, e, warp) : min_[RP > 1 ? e : 0];
-          return {v_add(l, h), v_sub(l, h)};
-        };
-        {
-          const PairSD<V> q = y_sums(Q19 ? 1 : 3);
-          f.a0 = v_add(f.a0, q.S);
-          f.jz = v_sub(f.jz, q.S);
-          f.rzz = v_add(f.rzz, q.S);
-          f.ryy = v_add(f.ryy, q.S);
-          f.jy = v_add(f.jy, q.D);
-          f.ryz = v_sub(f.ryz, q.D);
-          if constexpr (!Q19) {
-            const PairSD<V> q1 = y_sums(4);
-            f.jx = v_add(f.jx, q1.S);
-            f.rxz = v_sub(f.rxz, q1.S);
-            f.rxy = v_add(f.rxy, q1.D);
-            f.rxx = v_add(f.rxx, y_sums(5).S);
+          if (r == RP - 1 && warp < PAIRS - 1) {
+  #pragma unroll
+            for (int e = 0; e < NY; ++e) *y_at(it, 0, e, warp + 1) = P[e];
           }
+          if constexpr (RP > 1) {
+  #pragma unroll
+            for (int e = 0; e < NY; ++e) {
+              if (r == 0) pin[e] = P[e];
+              else min_[e] = M[e];
+            }
+          }
+          s0[r] = MASK && (in[r].e.l0 >> 31) != 0u;
+          s1[r] = MASK && (in[r].e.l1 >> 31) != 0u;
+          if constexpr (AHEAD) {
+            if (it + 1 < planes) fetch(in[r], it + 1);
+          }
+          // c_z = -1 part of the plane below, as far as it needs no neighbour row
+          Flight& f = fl[r];
+          f.rzz = v_add(MASK ? f.rzz : f.jz, own[r][3]);
+          f.a0 = v_add(f.a0, own[r][3]);
+          f.jz = v_sub(f.jz, own[r][3]);
+          f.jx = v_add(f.jx, own[r][4]);
+          f.rxz = v_sub(f.rxz, own[r][4]);
+          f.rxx = v_add(f.rxx, own[r][5]);
         }
-        if (it >= 2) {
-          const int z = z0 + it - 2;
-          // the sums are in units of the smallest weight, 1/36 or 1/216. p* and u, which accumulate over the steps,
-          // take that factor in two parts (rounded, and what it lacks): rounded once, it would scale them by
-          // 1 + 7e-9 (FP64 1 + 6e-17) in every step (FP32, 20 steps: error of u 9.1e-8 against 1.5e-7 with rounded
-          // weights; FP64, 50 steps, against 80-bit arithmetic: 3.2e-16 against 2.6e-15, for 1.5% of a 32^3 step)
-          constexpr T sc = Q19 ? T(1) / T(36) : T(1) / T(216);
-          // every term is exact: sc times powers of two, and differences of numbers within a factor of two
-          constexpr T lack = Q19 ? (T(1) - T(32) * sc - T(4) * sc) / T(36)
-                                 : (T(1) - T(128) * sc - T(64) * sc - T(16) * sc - T(8) * sc) / T(216);
-          const V vs = v_set<V>(sc), vl = v_set<V>(lack);
-          auto scaled = [&](V v) -> V { return v_fma(v, vs, v_mul(v, vl)); };
-          const V b0 = scaled(f.a0);
-          const bool own_row = ybl + warp * RP + r < yrows;
-          const bool w0 = own_row && gx >= xb && gx < nx && !f.sol0;
-          const bool w1 = VX == 2 && own_row && gx >= xb && gx + 1 < nx && !f.sol1;
-          const long long zc = (long long)z * plane + in[r].t.o0;
-          V hx_, hy_, hz_;
-          if constexpr (TWO != 0) {
-            V Fn[3] = {f.n0[0], f.n0[1], f.n0[2]};
-            if constexpr (TWO == 2) {
-              // density contrast (Sec. 2 force split): the force of the new state adds to F^s + F^b
-              //   F^p = -p* cs2 grad rho and F^nu = -(nu omega / cs2) a*_neq . grad rho,
-              // with p* = a*0 and a*_neq = a*2 - a*1 a*1 the raw moments just streamed in
-              const V jx_ = scaled(f.jx), jy_ = scaled(f.jy), jz_ = scaled(f.jz);
-              const V dr = v_set<V>(drho), gr0 = v_mul(f.ng[0], dr), gr1 = v_mul(f.ng[1], dr), gr2 = v_mul(f.ng[2], dr);
-              const V p3 = v_mul(b0, v_set<V>(T(1) / T(3)));
-              const V qxx = v_nfma(jx_, jx_, v_sub(v_mul(f.rxx, vs), p3));
-              const V qyy = v_nfma(jy_, jy_, v_sub(v_mul(f.ryy, vs), p3));
-              const V qzz = v_nfma(jz_, jz_, v_sub(v_mul(f.rzz, vs), p3));
-              const V qxy = v_nfma(jx_, jy_, v_mul(f.rxy, vs)), qxz = v_nfma(jx_, jz_, v_mul(f.rxz, vs));
-              const V qyz = v_nfma(jy_, jz_, v_mul(f.ryz, vs));
-              const V cnu = each(f.np[0], [&](T p) {
-                const T nu = nu_l + p * dnu;
-                return T(-3) * nu / (T(3) * nu + T(0.5));
-              });
-              Fn[0] = v_add(Fn[0], v_nfma(p3, gr0, v_mul(cnu, v_fma(qxx, gr0, v_fma(qxy, gr1, v_mul(qxz, gr2))))));
-              Fn[1] = v_add(Fn[1], v_nfma(p3, gr1, v_mul(cnu, v_fma(qxy, gr0, v_fma(qyy, gr1, v_mul(qyz, gr2))))));
-              Fn[2] = v_add(Fn[2], v_nfma(p3, gr2, v_mul(cnu, v_fma(qxz, gr0, v_fma(qyz, gr1, v_mul(qzz, gr2))))));
-              T* Fw = static_cast<T*>(a.F_new) + (long long)z * plane;
-#pragma unroll
-              for (int k = 0; k < 3; ++k) {
-                if constexpr (VX == 2) {
-                  if (w0) Fw[k * N + in[r].t.o0] = Fn[k].x;
-                  if (w1) Fw[k * N + in[r].t.o1] = Fn[k].y;
-                } else {
-                  if (w0) Fw[k * N + in[r].t.o0] = Fn[k];
+        if constexpr (TMA) {
+          bulk_wait_group_read0();  // the last outputs have left their stage
+        } else {
+  #pragma unroll
+          for (int r = 0; r < RP; ++r) copy_row(in[r], it - 1 + STAGES);  // into the stage of plane it - 1
+          copies_group();
+        }
+        cta_barrier<G::THREADS>();
+  #pragma unroll
+        for (int r = 0; r < RP; ++r) {
+          Flight& f = fl[r];
+          const int row = in[r].t.row;
+          auto y_sums = [&](int e) -> PairSD<V> {
+            const V l = r == 0 ? *y_at(it, 0, e, warp) : pin[RP > 1 ? e : 0];
+            const V h = r == RP - 1 ? *y_at(it, 1, e, warp) : min_[RP > 1 ? e : 0];
+            return {v_add(l, h), v_sub(l, h)};
+          };
+          {
+            const PairSD<V> q = y_sums(Q19 ? 1 : 3);
+            f.a0 = v_add(f.a0, q.S);
+            f.jz = v_sub(f.jz, q.S);
+            f.rzz = v_add(f.rzz, q.S);
+            f.ryy = v_add(f.ryy, q.S);
+            f.jy = v_add(f.jy, q.D);
+            f.ryz = v_sub(f.ryz, q.D);
+            if constexpr (!Q19) {
+              const PairSD<V> q1 = y_sums(4);
+              f.jx = v_add(f.jx, q1.S);
+              f.rxz = v_sub(f.rxz, q1.S);
+              f.rxy = v_add(f.rxy, q1.D);
+              f.rxx = v_add(f.rxx, y_sums(5).S);
+            }
+          }
+          if (it >= 2) {
+            const int z = z0 + it - 2;
+            // the sums are in units of the smallest weight, 1/36 or 1/216. p* and u, which accumulate over the steps,
+            // take that factor in two parts (rounded, and what it lacks): rounded once, it would scale them by
+            // 1 + 7e-9 (FP64 1 + 6e-17) in every step (FP32, 20 steps: error of u 9.1e-8 against 1.5e-7 with rounded
+            // weights; FP64, 50 steps, against 80-bit arithmetic: 3.2e-16 against 2.6e-15, for 1.5% of a 32^3 step)
+            constexpr T sc = Q19 ? T(1) / T(36) : T(1) / T(216);
+            // every term is exact: sc times powers of two, and differences of numbers within a factor of two
+            constexpr T lack = Q19 ? (T(1) - T(32) * sc - T(4) * sc) / T(36)
+                                   : (T(1) - T(128) * sc - T(64) * sc - T(16) * sc - T(8) * sc) / T(216);
+            const V vs = v_set<V>(sc), vl = v_set<V>(lack);
+            auto scaled = [&](V v) -> V { return v_fma(v, vs, v_mul(v, vl)); };
+            const V b0 = scaled(f.a0);
+            const bool own_row = ybl + warp * RP + r < yrows;
+            const bool w0 = own_row && gx >= xb && gx < nx && !f.sol0;
+            const bool w1 = VX == 2 && own_row && gx >= xb && gx + 1 < nx && !f.sol1;
+            const long long zc = (long long)z * plane + in[r].t.o0;
+            V hx_, hy_, hz_;
+            if constexpr (TWO != 0) {
+              V Fn[3] = {f.n0[0], f.n0[1], f.n0[2]};
+              if constexpr (TWO == 2) {
+                // density contrast (Sec. 2 force split): the force of the new state adds to F^s + F^b
+                //   F^p = -p* cs2 grad rho and F^nu = -(nu omega / cs2) a*_neq . grad rho,
+                // with p* = a*0 and a*_neq = a*2 - a*1 a*1 the raw moments just streamed in
+                const V jx_ = scaled(f.jx), jy_ = scaled(f.jy), jz_ = scaled(f.jz);
+                const V dr = v_set<V>(drho), gr0 = v_mul(f.ng[0], dr), gr1 = v_mul(f.ng[1], dr), gr2 = v_mul(f.ng[2], dr);
+                const V p3 = v_mul(b0, v_set<V>(T(1) / T(3)));
+                const V qxx = v_nfma(jx_, jx_, v_sub(v_mul(f.rxx, vs), p3));
+                const V qyy = v_nfma(jy_, jy_, v_sub(v_mul(f.ryy, vs), p3));
+                const V qzz = v_nfma(jz_, jz_, v_sub(v_mul(f.rzz, vs), p3));
+                const V qxy = v_nfma(jx_, jy_, v_mul(f.rxy, vs)), qxz = v_nfma(jx_, jz_, v_mul(f.rxz, vs));
+                const V qyz = v_nfma(jy_, jz_, v_mul(f.ryz, vs));
+                const V cnu = each(f.np[0], [&](T p) {
+                  const T nu = nu_l + p * dnu;
+                  return T(-3) * nu / (T(3) * nu + T(0.5));
+                });
+                Fn[0] = v_add(Fn[0], v_nfma(p3, gr0, v_mul(cnu, v_fma(qxx, gr0, v_fma(qxy, gr1, v_mul(qxz, gr2))))));
+                Fn[1] = v_add(Fn[1], v_nfma(p3, gr1, v_mul(cnu, v_fma(qxy, gr0, v_fma(qyy, gr1, v_mul(qyz, gr2))))));
+                Fn[2] = v_add(Fn[2], v_nfma(p3, gr2, v_mul(cnu, v_fma(qxz, gr0, v_fma(qyz, gr1, v_mul(qzz, gr2))))));
+                T* Fw = static_cast<T*>(a.F_new) + (long long)z * plane;
+  #pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                  if constexpr (VX == 2) {
+                    if (w0) Fw[k * N + in[r].t.o0] = Fn[k].x;
+                    if (w1) Fw[k * N + in[r].t.o1] = Fn[k].y;
+                  } else {
+                    if (w0) Fw[k * N + in[r].t.o0] = Fn[k];
+                  }
                 }
               }
-            }
-            const V hr = v_mul(rrho_of(f.np[0]), v_set<V>(T(0.5)));
-            hx_ = v_mul(Fn[0], hr), hy_ = v_mul(Fn[1], hr), hz_ = v_mul(Fn[2], hr);
-          } else if constexpr (FF)
-            hx_ = f.hx, hy_ = f.hy, hz_ = f.hz;
-          else
-            hx_ = v_set<V>(T(0.5) * Fu0), hy_ = v_set<V>(T(0.5) * Fu1), hz_ = v_set<V>(T(0.5) * Fu2);
-          // Eq. (corr), rho = 1: u = a1 + h with h = F/2, a2 = (sum c c f - cs2 a0 delta) + u h + h u, so
-          // N = a2 - u u = (sum c c f - cs2 a0 delta) - a1 a1 + h h
-          const V vx = scaled(f.jx), vy = scaled(f.jy), vz = scaled(f.jz);
-          const V ux = v_add(vx, hx_), uy = v_add(vy, hy_), uz = v_add(vz, hz_);
-          const V third = v_set<V>(T(-1) / T(3));
-          const V nxx = v_nfma(vx, vx, v_fma(f.rxx, vs, v_fma(b0, third, v_mul(hx_, hx_))));
-          const V nyy = v_nfma(vy, vy, v_fma(f.ryy, vs, v_fma(b0, third, v_mul(hy_, hy_))));
-          const V nzz = v_nfma(vz, vz, v_fma(f.rzz, vs, v_fma(b0, third, v_mul(hz_, hz_))));
-          const V nxy = v_nfma(vx, vy, v_fma(f.rxy, vs, v_mul(hx_, hy_)));
-          const V nxz = v_nfma(vx, vz, v_fma(f.rxz, vs, v_mul(hx_, hz_)));
-          const V nyz = v_nfma(vy, vz, v_fma(f.ryz, vs, v_mul(hy_, hz_)));
-          const V uu = v_fma(ux, ux, v_fma(uy, uy, v_mul(uz, uz)));
-          LBF_CHECK(a.flags, !(w0 || w1) || (z >= 0 && z < a.nz && in[r].t.o0 >= 0 && in[r].t.o0 < plane && zc + 9 * N < 10 * N));
-          S* d0 = dst + zc;
-          const T um = T(a.umax2);
-          if constexpr (VX == 2) {
-            uint32_t r0 = 0u, r1 = 0u;
-            if constexpr (Codec<S>::scaled && !RN) {
-              r0 = fmix32(uint32_t(zc) ^ a.salt);
-              r1 = fmix32(uint32_t(zc + 1) ^ a.salt);
-            }
-            if (by_tma) {
-              S* o = reinterpret_cast<S*>(stage_row(it, row)) + VX * lane;
-              st_pair<S, RN>(o, b0, a.sc.enc[0], r0, r1);
-              st_pair<S, RN>(o + XO, ux, a.sc.enc[1], r0, r1);
-              st_pair<S, RN>(o + 2 * XO, uy, a.sc.enc[1], r0, r1);
-              st_pair<S, RN>(o + 3 * XO, uz, a.sc.enc[1], r0, r1);
-              st_pair<S, true>(o + 4 * XO, nxx, a.sc.enc[2], r0, r1);
-              st_pair<S, true>(o + 5 * XO, nyy, a.sc.enc[2], r0, r1);
-              st_pair<S, true>(o + 6 * XO, nzz, a.sc.enc[2], r0, r1);
-              st_pair<S, true>(o + 7 * XO, nxy, a.sc.enc[2], r0, r1);
-              st_pair<S, true>(o + 8 * XO, nxz, a.sc.enc[2], r0, r1);
-              st_pair<S, true>(o + 9 * XO, nyz, a.sc.enc[2], r0, r1);
-              fence_proxy_async_smem();
-              __syncwarp();
-              if (r == RP - 1 && lane == 0) {
-                tma_store_4d(&tout, stage_row(it, row - r), x0, 0, gy[0], z);
-                bulk_commit_group();
+              const V hr = v_mul(rrho_of(f.np[0]), v_set<V>(T(0.5)));
+              hx_ = v_mul(Fn[0], hr), hy_ = v_mul(Fn[1], hr), hz_ = v_mul(Fn[2], hr);
+            } else if constexpr (FF)
+              hx_ = f.hx, hy_ = f.hy, hz_ = f.hz;
+            else
+              hx_ = v_set<V>(T(0.5) * Fu0), hy_ = v_set<V>(T(0.5) * Fu1), hz_ = v_set<V>(T(0.5) * Fu2);
+            // Eq. (corr), rho = 1: u = a1 + h with h = F/2, a2 = (sum c c f - cs2 a0 delta) + u h + h u, so
+            // N = a2 - u u = (sum c c f - cs2 a0 delta) - a1 a1 + h h
+            const V vx = scaled(f.jx), vy = scaled(f.jy), vz = scaled(f.jz);
+            const V ux = v_add(vx, hx_), uy = v_add(vy, hy_), uz = v_add(vz, hz_);
+            const V third = v_set<V>(T(-1) / T(3));
+            const V nxx = v_nfma(vx, vx, v_fma(f.rxx, vs, v_fma(b0, third, v_mul(hx_, hx_))));
+            const V nyy = v_nfma(vy, vy, v_fma(f.ryy, vs, v_fma(b0, third, v_mul(hy_, hy_))));
+            const V nzz = v_nfma(vz, vz, v_fma(f.rzz, vs, v_fma(b0, third, v_mul(hz_, hz_))));
+            const V nxy = v_nfma(vx, vy, v_fma(f.rxy, vs, v_mul(hx_, hy_)));
+            const V nxz = v_nfma(vx, vz, v_fma(f.rxz, vs, v_mul(hx_, hz_)));
+            const V nyz = v_nfma(vy, vz, v_fma(f.ryz, vs, v_mul(hy_, hz_)));
+            const V uu = v_fma(ux, ux, v_fma(uy, uy, v_mul(uz, uz)));
+            LBF_CHECK(a.flags, !(w0 || w1) || (z >= 0 && z < a.nz && in[r].t.o0 >= 0 && in[r].t.o0 < plane && zc + 9 * N < 10 * N));
+            S* d0 = dst + zc;
+            const T um = T(a.umax2);
+            if constexpr (VX == 2) {
+              uint32_t r0 = 0u, r1 = 0u;
+              if constexpr (Codec<S>::scaled && !RN) {
+                r0 = fmix32(uint32_t(zc) ^ a.salt);
+                r1 = fmix32(uint32_t(zc + 1) ^ a.salt);
               }
-            } else if (TMA && w0 && w1) {
-              st_pair<S, RN>(d0, b0, a.sc.enc[0], r0, r1);
-              st_pair<S, RN>(d0 + N, ux, a.sc.enc[1], r0, r1);
-              st_pair<S, RN>(d0 + 2 * N, uy, a.sc.enc[1], r0, r1);
-              st_pair<S, RN>(d0 + 3 * N, uz, a.sc.enc[1], r0, r1);
-              st_pair<S, true>(d0 + 4 * N, nxx, a.sc.enc[2], r0, r1);
-              st_pair<S, true>(d0 + 5 * N, nyy, a.sc.enc[2], r0, r1);
-              st_pair<S, true>(d0 + 6 * N, nzz, a.sc.enc[2], r0, r1);
-              st_pair<S, true>(d0 + 7 * N, nxy, a.sc.enc[2], r0, r1);
-              st_pair<S, true>(d0 + 8 * N, nxz, a.sc.enc[2], r0, r1);
-              st_pair<S, true>(d0 + 9 * N, nyz, a.sc.enc[2], r0, r1);
-            } else if (!TMA || MASK) {
-              auto put = [&](int at, uint32_t& rr, float p_, float x_, float y_, float z_, float xx, float yy, float zz,
-                             float xy, float xz, float yz) {
-                S* d = d0 + at;
-                st_field<S, RN>(d, 0, p_, a.sc.enc[0], rr);
-                st_field<S, RN>(d + N, 0, x_, a.sc.enc[1], rr);
-                st_field<S, RN>(d + 2 * N, 0, y_, a.sc.enc[1], rr);
-                st_field<S, RN>(d + 3 * N, 0, z_, a.sc.enc[1], rr);
-                st_field<S, true>(d + 4 * N, 0, xx, a.sc.enc[2], rr);
-                st_field<S, true>(d + 5 * N, 0, yy, a.sc.enc[2], rr);
-                st_field<S, true>(d + 6 * N, 0, zz, a.sc.enc[2], rr);
-                st_field<S, true>(d + 7 * N, 0, xy, a.sc.enc[2], rr);
-                st_field<S, true>(d + 8 * N, 0, xz, a.sc.enc[2], rr);
-                st_field<S, true>(d + 9 * N, 0, yz, a.sc.enc[2], rr);
-              };
-              if (w0) put(0, r0, b0.x, ux.x, uy.x, uz.x, nxx.x, nyy.x, nzz.x, nxy.x, nxz.x, nyz.x);
-              if (w1) put(1, r1, b0.y, ux.y, uy.y, uz.y, nxx.y, nyy.y, nzz.y, nxy.y, nxz.y, nyz.y);
+              if (by_tma) {
+                S* o = reinterpret_cast<S*>(stage_row(it, row)) + VX * lane;
+                st_pair<S, RN>(o, b0, a.sc.enc[0], r0, r1);
+                st_pair<S, RN>(o + XO, ux, a.sc.enc[1], r0, r1);
+                st_pair<S, RN>(o + 2 * XO, uy, a.sc.enc[1], r0, r1);
+                st_pair<S, RN>(o + 3 * XO, uz, a.sc.enc[1], r0, r1);
+                st_pair<S, true>(o + 4 * XO, nxx, a.sc.enc[2], r0, r1);
+                st_pair<S, true>(o + 5 * XO, nyy, a.sc.enc[2], r0, r1);
+                st_pair<S, true>(o + 6 * XO, nzz, a.sc.enc[2], r0, r1);
+                st_pair<S, true>(o + 7 * XO, nxy, a.sc.enc[2], r0, r1);
+                st_pair<S, true>(o + 8 * XO, nxz, a.sc.enc[2], r0, r1);
+                st_pair<S, true>(o + 9 * XO, nyz, a.sc.enc[2], r0, r1);
+                fence_proxy_async_smem();
+                __syncwarp();
+                if (r == RP - 1 && lane == 0) {
+                  tma_store_4d(&tout, stage_row(it, row - r), x0, 0, gy[0], z);
+                  bulk_commit_group();
+                }
+              } else if (TMA && w0 && w1) {
+                st_pair<S, RN>(d0, b0, a.sc.enc[0], r0, r1);
+                st_pair<S, RN>(d0 + N, ux, a.sc.enc[1], r0, r1);
+                st_pair<S, RN>(d0 + 2 * N, uy, a.sc.enc[1], r0, r1);
+                st_pair<S, RN>(d0 + 3 * N, uz, a.sc.enc[1], r0, r1);
+                st_pair<S, true>(d0 + 4 * N, nxx, a.sc.enc[2], r0, r1);
+                st_pair<S, true>(d0 + 5 * N, nyy, a.sc.enc[2], r0, r1);
+                st_pair<S, true>(d0 + 6 * N, nzz, a.sc.enc[2], r0, r1);
+                st_pair<S, true>(d0 + 7 * N, nxy, a.sc.enc[2], r0, r1);
+                st_pair<S, true>(d0 + 8 * N, nxz, a.sc.enc[2], r0, r1);
+                st_pair<S, true>(d0 + 9 * N, nyz, a.sc.enc[2], r0, r1);
+              } else if (!TMA || MASK) {
+                auto put = [&](int at, uint32_t& rr, float p_, float x_, float y_, float z_, float xx, float yy, float zz,
+                               float xy, float xz, float yz) {
+                  S* d = d0 + at;
+                  st_field<S, RN>(d, 0, p_, a.sc.enc[0], rr);
+                  st_field<S, RN>(d + N, 0, x_, a.sc.enc[1], rr);
+                  st_field<S, RN>(d + 2 * N, 0, y_, a.sc.enc[1], rr);
+                  st_field<S, RN>(d + 3 * N, 0, z_, a.sc.enc[1], rr);
+                  st_field<S, true>(d + 4 * N, 0, xx, a.sc.enc[2], rr);
+                  st_field<S, true>(d + 5 * N, 0, yy, a.sc.enc[2], rr);
+                  st_field<S, true>(d + 6 * N, 0, zz, a.sc.enc[2], rr);
+                  st_field<S, true>(d + 7 * N, 0, xy, a.sc.enc[2], rr);
+                  st_field<S, true>(d + 8 * N, 0, xz, a.sc.enc[2], rr);
+                  st_field<S, true>(d + 9 * N, 0, yz, a.sc.enc[2], rr);
+                };
+                if (w0) put(0, r0, b0.x, ux.x, uy.x, uz.x, nxx.x, nyy.x, nzz.x, nxy.x, nxz.x, nyz.x);
+                if (w1) put(1, r1, b0.y, ux.y, uy.y, uz.y, nxx.y, nyy.y, nzz.y, nxy.y, nxz.y, nyz.y);
+              }
+              bad = bad || (w0 && !(uu.x <= um)) || (w1 && !(uu.y <= um));
+              if (a.partials != nullptr) {
+                red[0] += (w0 ? b0.x : 0.0f) + (w1 ? b0.y : 0.0f);
+                red[1] += (w0 ? ux.x : 0.0f) + (w1 ? ux.y : 0.0f);
+                red[2] += (w0 ? uy.x : 0.0f) + (w1 ? uy.y : 0.0f);
+                red[3] += (w0 ? uz.x : 0.0f) + (w1 ? uz.y : 0.0f);
+                if constexpr (TWO != 0) red[4] += (w0 ? f.np[0].x : 0.0f) + (w1 ? f.np[0].y : 0.0f);
+                red[5] += (w0 ? uu.x : 0.0f) + (w1 ? uu.y : 0.0f);
+              }
+            } else if (w0) {
+              d0[0] = b0;
+              d0[N] = ux;
+              d0[2 * N] = uy;
+              d0[3 * N] = uz;
+              d0[4 * N] = nxx;
+              d0[5 * N] = nyy;
+              d0[6 * N] = nzz;
+              d0[7 * N] = nxy;
+              d0[8 * N] = nxz;
+              d0[9 * N] = nyz;
+              bad = bad || !(uu <= um);
+              red[0] += b0;
+              red[1] += ux;
+              red[2] += uy;
+              red[3] += uz;
+              if constexpr (TWO != 0) red[4] += f.np[0];
+              red[5] += uu;
             }
-            bad = bad || (w0 && !(uu.x <= um)) || (w1 && !(uu.y <= um));
-            if (a.partials != nullptr) {
-              red[0] += (w0 ? b0.x : 0.0f) + (w1 ? b0.y : 0.0f);
-              red[1] += (w0 ? ux.x : 0.0f) + (w1 ? ux.y : 0.0f);
-              red[2] += (w0 ? uy.x : 0.0f) + (w1 ? uy.y : 0.0f);
-              red[3] += (w0 ? uz.x : 0.0f) + (w1 ? uz.y : 0.0f);
-              if constexpr (TWO != 0) red[4] += (w0 ? f.np[0].x : 0.0f) + (w1 ? f.np[0].y : 0.0f);
-              red[5] += (w0 ? uu.x : 0.0f) + (w1 ? uu.y : 0.0f);
+          }
+          fetch_new(in[r], f, it);
+          // this plane becomes the one in flight: c_z = +1 of the plane below plus its own c_z = 0 part
+          auto mid = [&](V u, V v) { return Q19 ? v_add(u, v) : v_fma(v, v_set<V>(T(4)), u); };
+          {
+            const PairSD<V> q0 = y_sums(Q19 ? 2 : 6), q1 = y_sums(Q19 ? 3 : 7);
+            f.a0 = mid(f.u00, v_add(own[r][6], q0.S));
+            f.ryy = mid(f.u02, q0.S);
+            f.jy = mid(f.u01, q0.D);
+            f.jx = mid(f.u10, v_add(own[r][7], q1.S));
+            f.rxy = Q19 ? q1.D : mid(f.u11, q1.D);
+            f.rxx = mid(f.u20, v_add(own[r][8], y_sums(Q19 ? 4 : 8).S));
+          }
+          f.jz = f.u00;
+          f.rxz = f.u10;
+          f.ryz = f.u01;
+          if constexpr (MASK) {
+            f.rzz = f.u00;
+            if (dirty) {
+              const V* const b = cor_at(it, row);
+              f.a0 = v_add(f.a0, b[0]);
+              f.jx = v_add(f.jx, b[32]);
+              f.jy = v_add(f.jy, b[2 * 32]);
+              f.jz = v_add(f.jz, b[3 * 32]);
+              f.rxx = v_add(f.rxx, b[4 * 32]);
+              f.ryy = v_add(f.ryy, b[5 * 32]);
+              f.rzz = v_add(f.rzz, b[6 * 32]);
+              f.rxy = v_add(f.rxy, b[7 * 32]);
+              f.rxz = v_add(f.rxz, b[8 * 32]);
+              f.ryz = v_add(f.ryz, b[9 * 32]);
             }
-          } else if (w0) {
-            d0[0] = b0;
-            d0[N] = ux;
-            d0[2 * N] = uy;
-            d0[3 * N] = uz;
-            d0[4 * N] = nxx;
-            d0[5 * N] = nyy;
-            d0[6 * N] = nzz;
-            d0[7 * N] = nxy;
-            d0[8 * N] = nxz;
-            d0[9 * N] = nyz;
-            bad = bad || !(uu <= um);
-            red[0] += b0;
-            red[1] += ux;
-            red[2] += uy;
-            red[3] += uz;
-            if constexpr (TWO != 0) red[4] += f.np[0];
-            red[5] += uu;
+            f.sol0 = s0[r];
+            f.sol1 = s1[r];
           }
-        }
-        fetch_new(in[r], f, it);
-        // this plane becomes the one in flight: c_z = +1 of the plane below plus its own c_z = 0 part
-        auto mid = [&](V u, V v) { return Q19 ? v_add(u, v) : v_fma(v, v_set<V>(T(4)), u); };
-        {
-          const PairSD<V> q0 = y_sums(Q19 ? 2 : 6), q1 = y_sums(Q19 ? 3 : 7);
-          f.a0 = mid(f.u00, v_add(own[r][6], q0.S));
-          f.ryy = mid(f.u02, q0.S);
-          f.jy = mid(f.u01, q0.D);
-          f.jx = mid(f.u10, v_add(own[r][7], q1.S));
-          f.rxy = Q19 ? q1.D : mid(f.u11, q1.D);
-          f.rxx = mid(f.u20, v_add(own[r][8], y_sums(Q19 ? 4 : 8).S));
-        }
-        f.jz = f.u00;
-        f.rxz = f.u10;
-        f.ryz = f.u01;
-        if constexpr (MASK) {
-          f.rzz = f.u00;
-          if (dirty) {
-            const V* const b = cor_at(it, row);
-            f.a0 = v_add(f.a0, b[0]);
-            f.jx = v_add(f.jx, b[32]);
-            f.jy = v_add(f.jy, b[2 * 32]);
-            f.jz = v_add(f.jz, b[3 * 32]);
-            f.rxx = v_add(f.rxx, b[4 * 32]);
-            f.ryy = v_add(f.ryy, b[5 * 32]);
-            f.rzz = v_add(f.rzz, b[6 * 32]);
-            f.rxy = v_add(f.rxy, b[7 * 32]);
-            f.rxz = v_add(f.rxz, b[8 * 32]);
-            f.ryz = v_add(f.ryz, b[9 * 32]);
+          if constexpr (FF) {
+            const V half = v_set<V>(T(0.5));
+            f.hx = v_mul(F[r][0], half), f.hy = v_mul(F[r][1], half), f.hz = v_mul(F[r][2], half);
           }
-          f.sol0 = s0[r];
-          f.sol1 = s1[r];
-        }
-        if constexpr (FF) {
-          const V half = v_set<V>(T(0.5));
-          f.hx = v_mul(F[r][0], half), f.hy = v_mul(F[r][1], half), f.hz = v_mul(F[r][2], half);
-        }
-        {
-          const PairSD<V> q = y_sums(0);
-          f.u00 = v_add(own[r][0], q.S);
-          f.u02 = q.S;
-          f.u01 = q.D;
-          if constexpr (Q19) {
-            f.u10 = own[r][1];
-            f.u20 = own[r][2];
-          } else {
-            const PairSD<V> q1 = y_sums(1);
-            f.u10 = v_add(own[r][1], q1.S);
-            f.u11 = q1.D;
-            f.u20 = v_add(own[r][2], y_sums(2).S);
+          {
+            const PairSD<V> q = y_sums(0);
+            f.u00 = v_add(own[r][0], q.S);
+            f.u02 = q.S;
+            f.u01 = q.D;
+            if constexpr (Q19) {
+              f.u10 = own[r][1];
+              f.u20 = own[r][2];
+            } else {
+              const PairSD<V> q1 = y_sums(1);
+              f.u10 = v_add(own[r][1], q1.S);
+              f.u11 = q1.D;
+              f.u20 = v_add(own[r][2], y_sums(2).S);
+            }
           }
         }
       }
-    }
+      if constexpr (PARTS) {
+        if (a.partials != nullptr) {
+#pragma unroll
+          for (int k = 0; k < 6; ++k) {
+            const double v = warp_sum(red[k]);
+            if (lane == 0) parts[warp * 6 + k] += v;
+            red[k] = T(0);
+          }
+        }
+      }
+    } while (PARTS && it < planes && !gave_up[(it - 1) & 1]);
     if constexpr (TMA) bulk_wait_group0();
     else asm volatile("cp.async.wait_all;" ::: "memory");
     if (bad) atomicOr(a.flags, 1u);
@@ -1296,17 +1322,17 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
   grid_release();
 
   if (a.partials != nullptr) {
-    // warp sums in the compute type, block and grid sums in FP64, in a fixed order
-    double* red_s = reinterpret_cast<double*>(sbase);
+    // warp sums (of some planes) in the compute type, the others in FP64, in a fixed order
+    double* red_s = PARTS ? parts : reinterpret_cast<double*>(sbase);
     const int tid = warp * 32 + lane;
+    if constexpr (!PARTS) {
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      T v = red[k];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) red_s[warp * 6 + k] = static_cast<double>(v);
+      for (int k = 0; k < 6; ++k) {
+        const double v = warp_sum(red[k]);
+        if (lane == 0) red_s[warp * 6 + k] = v;
+      }
+      __syncthreads();
     }
-    __syncthreads();
     const long long nb = (long long)gridDim.x * gridDim.y * gridDim.z;
     if (tid < 6) {
       double s = 0.0;
