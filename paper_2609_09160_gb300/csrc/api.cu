@@ -133,6 +133,22 @@ bool sep_built(const lbf_params* p) {
   if (p->two_component) return p->lattice == LBF_D3Q19 && p->storage == LBF_F32;
   return !p->populations && !(p->lattice == LBF_D3Q27H && p->mask != nullptr);
 }
+// LBF_KERNEL names the step's kernel (tests, tuning)
+std::string kernel_name() {
+  const char* kind = std::getenv("LBF_KERNEL");
+  return kind ? kind : "";
+}
+bool sep_forced(const std::string& kname) { return kname == "sep" || kname == "sepsmall"; }
+// sites below which the axis-separated kernel takes its short tile, and walls of any shape
+constexpr long long kSepSmall = 1LL << 20;
+// its masked form, the only user of the wall links and tile flags: walls with two components, on small lattices, or
+// by name. (Larger lattices are split into clean rows and rows near walls, or take the 30-column kernel)
+bool sep_masked(const lbf_params* p, const std::string& kname) {
+  if (p->mask == nullptr || !sep_built(p)) return false;
+  if (sep_forced(kname)) return true;
+  const bool small = (long long)p->nx * p->ny * p->nz < kSepSmall && storage_bytes(p->storage) != 2;
+  return kname.empty() && (p->two_component || small);
+}
 // z-chunks of the axis-separated kernel: at most kSepMaxZ planes (64 with one FP32 row per warp, whose threads add
 // up their sums over a whole chunk), at least two and no fewer than keep a grid of `tiles` columns within
 // kSepBlocks blocks (one 64-byte partial sum each) where that is possible
@@ -173,7 +189,7 @@ bool make_layout(const lbf_params* p, Layout* L) {
   L->state[1] = take(fields * N * sb);
   L->mom = p->populations ? take(10 * N * sb) : 0;
   L->mask = p->mask ? take(N) : 0;
-  const bool links = p->mask != nullptr && sep_built(p);
+  const bool links = sep_masked(p, kernel_name());
   L->links = links ? take(N * sizeof(uint32_t)) : 0;
   L->dirty = links ? take(sep_max_tiles(p)) : 0;
   if (p->two_component) {
@@ -224,7 +240,7 @@ struct lbf_ctx {
   void* state[2];
   int cur;
   uint8_t* mask_d;
-  uint32_t* links_d;   // walls: per-site links and per-tile flags of the axis-separated kernel
+  uint32_t* links_d;   // walls: per-site links and per-tile flags of the axis-separated kernel's masked form
   uint8_t* dirty_d;
   void* phi[2];
   void* F[2];
@@ -775,7 +791,7 @@ lbf_status setup_split(lbf_ctx* c, const lbf_params* p, const Layout& L, int sms
 
 // Chooses the axis-separated kernel for the step, its tile and its z-chunk.
 lbf_status setup_sep(lbf_ctx* c, const lbf_params* p, const Layout& L, int sms, bool nearest, const std::string& kname) {
-  const bool forced = kname == "sep" || kname == "sepsmall";
+  const bool forced = sep_forced(kname);
   if (!sep_built(p) || !(kname.empty() || forced)) return LBF_OK;
   if (storage_bytes(c->storage) == 2 && c->nx % 2 != 0) return LBF_OK;  // no 4-byte aligned pairs of sites
   // 16-bit storage keeps the kernels whose roundings it has, with and without walls. A stored p* or u is the
@@ -788,7 +804,7 @@ lbf_status setup_sep(lbf_ctx* c, const lbf_params* p, const Layout& L, int sms, 
   const bool field = p->force_field != nullptr;
   // below about 2^20 sites the tall tiles leave SMs idle: short ones (ensemble members, 524288 sites with
   // walls and a force field: 17 us a step against 20.6)
-  const bool small = kname == "sepsmall" || (kname != "sep" && c->N < (1LL << 20));
+  const bool small = kname == "sepsmall" || (kname != "sep" && c->N < kSepSmall);
   const bool rows_tma = tma_eligible(c->storage, c->nx) && c->nx >= 32 * sep_vx(int(storage_bytes(c->storage)));
   // large lattices whose rows TMA cannot take: the 30-column kernel (333 x 250 x 189, GLUPS: 38.0 against
   // 34.8 with the best tile of this one)
@@ -815,6 +831,7 @@ lbf_status setup_sep(lbf_ctx* c, const lbf_params* p, const Layout& L, int sms, 
     c->zchunk_dirty = std::max(std::min(LBF_SEP_SPLIT_ZCHUNK, c->nz), grid_min_z(c->nz));
     c->grid_dirty = dim3(grid_x(c->nx, c->fwd.xout), grid_y(c->dirty_rows, c->fwd.by), (c->nz + c->zchunk_dirty - 1) / c->zchunk_dirty);
   }
+  if (walls && c->links_d == nullptr) return fail(LBF_EINTERNAL, "no room for the wall links");
   c->sep.async = kernel(false);
   c->sep.tma = KernelInfo{nullptr, 0, 0, 0, 0};
   if (rows_tma)
@@ -1185,8 +1202,7 @@ lbf_status lbf_create(lbf_ctx** out, const lbf_params* params, void* workspace, 
   // at 512^3, +8% at 256^3), periodic D3Q19 16-bit and D3Q27 FP32 on planes of at least 512 x 512
   // (+3%, +2% at 512^3); slower with walls, for D3Q27h and for 16-bit D3Q27. LBF_KERNEL=aligned or
   // cta forces one of them.
-  const char* kind = std::getenv("LBF_KERNEL");
-  const std::string kname = kind ? kind : "";
+  const std::string kname = kernel_name();
   const long long plane_sites = (long long)c->nx * c->ny;
   const bool q19_f32 = c->Q == LBF_D3Q19 && c->storage == LBF_F32;
   const bool large = plane_sites >= (q19_f32 ? 256LL * 256LL : 512LL * 512LL);
