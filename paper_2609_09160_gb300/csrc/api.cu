@@ -269,6 +269,7 @@ struct lbf_ctx {
   // 30-column kernel on the others (sep_split)
   struct {
     bool on;
+    bool ring;              // the clean rows of a split run the periodic 30-column kernel (row: its map)
     KernelInfo tma, async;  // rows by TMA (fn null where they do not allow it), or by cp.async
     CUtensorMap row[2], tile[2], out[2];  // maps of the two state buffers: load boxes of one row and of a
                                           // tile's rows, store boxes
@@ -636,6 +637,67 @@ int choose_zchunk_sep(int nz, long long tiles, double resident, double min_waves
   return zc;
 }
 
+// ---- which of two kernels a step takes: the one with the shorter estimate -------------------------------------
+// A CTA takes `lone` us a plane where it has its SM to itself (latency) and adds `busy` us to an SM that runs others
+// beside it (issue, FP64 pipe, shared memory), so k resident CTAs take max(lone, k busy) us a plane together; a launch
+// runs in rounds of `resident` CTAs per SM, and many rounds run into one another. Fitted to both kernels' times on
+// 1871 lattices (2^9 to 2^27 sites, every form below) on one GB300: the estimates are within 5 to 10% of the times, the
+// choice by them is 1.3% slower than always the faster kernel. Without it, the axis-separated kernel always, 769 of
+// them were slower than with the 30-column one: tiles of 64 (FP64 32) columns waste lanes on rows of other lengths,
+// force fields (D3Q19 FP32 256^3: 424 us against 340) and FP64 walls (12 x 64 x 64: 124 against 76) cost it more, and
+// D3Q27h in FP64 is arithmetic (256^3: 27.1 ms against 23.2).
+struct PlaneTime {
+  double lone, busy;
+};
+double estimate_us(long long blocks, int sms, int resident, double planes, PlaneTime p) {
+  const long long per_sm = (blocks + sms - 1) / sms, full = per_sm / resident, rest = per_sm % resident;
+  const double round = std::max(p.lone, p.busy * resident);
+  if (full >= 4) return planes * round * (double(blocks) / (double(sms) * resident) + 0.3);
+  return planes * (full * round + (rest > 0 ? std::max(p.lone, p.busy * rest) : 0.0));
+}
+// the 30-column kernel (two: 1 equal densities, 2 a density contrast)
+PlaneTime ring_plane(int lattice, int storage, bool walls, bool field, int two) {
+  if (storage == LBF_F64) {  // the FP64 pipe
+    const double t = (lattice == LBF_D3Q19 ? 7.2 : (lattice == LBF_D3Q27 ? 9.5 : 21.5)) * (field ? 1.04 : 1.0);
+    return {t, t};
+  }
+  if (two == 1) return walls ? PlaneTime{2.26, 1.13} : PlaneTime{1.63, 0.84};
+  if (two == 2) return walls ? PlaneTime{2.87, 1.40} : PlaneTime{1.93, 1.02};
+  PlaneTime p = {1.12, 0.76};  // D3Q27h
+  if (lattice == LBF_D3Q19) p = walls ? PlaneTime{1.0, 0.70} : PlaneTime{0.87, 0.60};
+  if (lattice == LBF_D3Q27) p = walls ? PlaneTime{1.22, 0.87} : PlaneTime{0.87, 0.54};
+  if (field) p = {1.07 * p.lone, 1.07 * p.busy};
+  return p;
+}
+// the axis-separated kernel: walls in its masked form, or the clean rows of a split step
+PlaneTime sep_plane(int lattice, int storage, bool walls, bool split, bool field, int two, bool small, bool rows_tma, int nx) {
+  PlaneTime p;
+  double f = 1.0;
+  if (storage == LBF_F64) {
+    const double t = lattice == LBF_D3Q19 ? (walls ? 5.1 : 3.7) : (lattice == LBF_D3Q27 ? (walls ? 6.7 : 5.0) : 14.0);
+    p = {t, t};
+    f = (field && !walls ? 1.13 : 1.0) * (rows_tma ? 1.0 : 1.08);
+  } else if (two != 0) {
+    p = two == 1 ? (walls ? PlaneTime{2.9, 1.65} : PlaneTime{2.44, 1.35}) : (walls ? PlaneTime{3.4, 2.1} : PlaneTime{2.7, 1.65});
+    f = rows_tma ? 1.0 : 1.25;
+  } else if (small) {
+    p = {1.14, 1.08};  // D3Q27h
+    if (lattice == LBF_D3Q19) p = walls ? PlaneTime{0.70, 0.62} : PlaneTime{0.45, 0.41};
+    if (lattice == LBF_D3Q27) p = walls ? PlaneTime{0.85, 0.74} : PlaneTime{0.58, 0.54};
+    f = field && !walls ? 1.2 : 1.0;
+    if (!rows_tma) f *= lattice == LBF_D3Q19 ? 1.5 : (lattice == LBF_D3Q27 ? 1.4 : 1.12);
+  } else {
+    p = {1.39, 1.39};  // D3Q27h
+    if (lattice == LBF_D3Q19) p = {1.0, 1.0};
+    if (lattice == LBF_D3Q27) p = {0.93, 0.57};
+    if (split) f = 1.05;
+    if (field) f *= lattice == LBF_D3Q19 ? 1.7 : (lattice == LBF_D3Q27 ? 1.6 : 1.25);
+  }
+  // rows of one or two FP32 sites: every lane copies the same few (900 x 900 planes of 1: 3209 us, the ring 321)
+  if (storage != LBF_F64 && nx < 4) f *= 4.0;
+  return {f * p.lone, f * p.busy};
+}
+
 // z-chunk of a launch of `tiles` x-y tiles: the CTAs of one tile column march through nz / chunks
 // planes each, restaging two planes per chunk. Large lattices: the longest chunk (16 to 64 planes)
 // that still gives at least kMinWaves waves of resident CTAs, since fewer, longer-lived CTAs start
@@ -732,6 +794,14 @@ bool clean_band(const lbf_ctx* c, const lbf_params* p, int by, int* begin, int* 
   return best_len >= ny / 2 && best_len >= 2 * by;
 }
 
+// whether setup_split (below) may split this lattice; any: of any plane size (LBF_KERNEL=split, tests)
+bool split_by_aligned(const lbf_ctx* c, const lbf_params* p, bool any = false) {
+  if (!c->has_mask || c->two || c->pops || !c->tma || c->aligned || p->force_field != nullptr || LBF_AL_TMA_STORE) return false;
+  const bool q19_f32 = c->Q == LBF_D3Q19 && c->storage == LBF_F32;
+  return (any || (long long)c->nx * c->ny >= (q19_f32 ? 256LL * 256LL : 512LL * 512LL)) &&
+         ((c->Q == LBF_D3Q19 && c->storage != LBF_F64) || (c->Q == LBF_D3Q27 && c->storage == LBF_F32));
+}
+
 // Row split for walls that occupy few rows (a channel's walls): row y is clean when rows y-1, y,
 // y+1 (periodic) hold no solid site at any x and z, so every population its outputs pull comes
 // from a fluid site and the periodic kernel (no mask logic) computes them exactly. When the clean
@@ -740,15 +810,7 @@ bool clean_band(const lbf_ctx* c, const lbf_params* p, int by, int* begin, int* 
 // the library picks for periodic lattices of this size and type and setup_sep did not take the lattice.
 lbf_status setup_split(lbf_ctx* c, const lbf_params* p, const Layout& L, int sms, bool nearest,
                        const std::string& kname) {
-  if (!c->has_mask || c->two || c->pops || !c->tma || c->aligned || p->force_field != nullptr || LBF_AL_TMA_STORE ||
-      kname == "cta" || kname == "aligned")
-    return LBF_OK;
-  const long long plane_sites = (long long)c->nx * c->ny;
-  const bool q19_f32 = c->Q == LBF_D3Q19 && c->storage == LBF_F32;
-  const bool forced = kname == "split";  // LBF_KERNEL=split: any plane size (tests)
-  if ((!forced && plane_sites < (q19_f32 ? 256LL * 256LL : 512LL * 512LL)) ||
-      !((c->Q == LBF_D3Q19 && c->storage != LBF_F64) || (c->Q == LBF_D3Q27 && c->storage == LBF_F32)))
-    return LBF_OK;
+  if (kname == "cta" || kname == "aligned" || !split_by_aligned(c, p, kname == "split")) return LBF_OK;
   const KernelInfo al = aligned_kernel_for(c->Q, c->storage, false, false, nearest);
   if (al.fn == nullptr) return LBF_OK;
   const int nx = c->nx, ny = c->ny, nz = c->nz;
@@ -787,6 +849,18 @@ lbf_status setup_split(lbf_ctx* c, const lbf_params* p, const Layout& L, int sms
   c->grid_dirty = gd;
   c->split = true;
   return LBF_OK;
+}
+
+// maps of a state buffer for the TMA kernel of c->sep: of its loads (one row, a tile's rows; with the 30-column
+// kernel its one box) and of its stores
+lbf_status sep_source_maps(const lbf_ctx* c, const void* base, CUtensorMap* row, CUtensorMap* tile) {
+  const KernelInfo& k = c->sep.tma;
+  if (c->sep.ring) return encode_state_map(c, base, row, k.box_x, k.by + 2);
+  const lbf_status st = encode_row_map(c, base, row, k.box_x, 1);
+  return st != LBF_OK ? st : encode_row_map(c, base, tile, k.box_x, k.by + 2);
+}
+lbf_status sep_store_map(const lbf_ctx* c, const void* base, CUtensorMap* out) {
+  return c->sep.ring ? LBF_OK : encode_row_map(c, base, out, c->sep.tma.box_x, c->sep.tma.out_rows);
 }
 
 // Chooses the axis-separated kernel for the step, its tile and its z-chunk.
@@ -832,34 +906,72 @@ lbf_status setup_sep(lbf_ctx* c, const lbf_params* p, const Layout& L, int sms, 
     c->grid_dirty = dim3(grid_x(c->nx, c->fwd.xout), grid_y(c->dirty_rows, c->fwd.by), (c->nz + c->zchunk_dirty - 1) / c->zchunk_dirty);
   }
   if (walls && c->links_d == nullptr) return fail(LBF_EINTERNAL, "no room for the wall links");
-  c->sep.async = kernel(false);
-  c->sep.tma = KernelInfo{nullptr, 0, 0, 0, 0};
-  if (rows_tma)
-    c->sep.tma = kernel(true);
   lbf_status st;
-  if ((st = prepare(c->sep.async)) != LBF_OK || (st = prepare(c->sep.tma)) != LBF_OK) return st;
-  const KernelInfo& k = c->sep.tma.fn ? c->sep.tma : c->sep.async;
   int resident = 1;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, k.fn, k.threads, k.smem) != cudaSuccess)
-    return fail(LBF_ECUDA, std::string("device query failed: ") + cudaGetErrorString(cudaGetLastError()));
-  const long long tiles = (long long)grid_x(c->nx, k.xout) * grid_y(c->sep.y_rows, k.by);
-  const int zmax = sep_max_z(k.out_rows, c->storage);
-  c->sep.zchunk = choose_zchunk_sep(c->nz, tiles, double(sms) * std::max(resident, 1), split ? 2.0 : 1.0, zmax);
-  if (const char* e = std::getenv("LBF_ZCHUNK")) {
-    const int v = std::atoi(e);
-    if (v >= 1) c->sep.zchunk = std::min({c->nz, zmax, std::max(sep_min_z(c->nz, tiles, zmax), v)});
-  }
-  c->sep.grid = dim3(grid_x(c->nx, k.xout), grid_y(c->sep.y_rows, k.by), (c->nz + c->sep.zchunk - 1) / c->sep.zchunk);
+  // takes the kernels of this step, the z-chunk that `choose` gives for (tiles, resident CTAs), and their grid
+  auto take = [&](const KernelInfo& by_tma, const KernelInfo& other, auto choose) -> lbf_status {
+    c->sep.tma = by_tma;
+    c->sep.async = other;
+    if ((st = prepare(by_tma)) != LBF_OK || (st = prepare(other)) != LBF_OK) return st;
+    const KernelInfo& k = by_tma.fn ? by_tma : other;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, k.fn, k.threads, k.smem) != cudaSuccess)
+      return fail(LBF_ECUDA, std::string("device query failed: ") + cudaGetErrorString(cudaGetLastError()));
+    resident = std::max(resident, 1);
+    const long long tiles = (long long)grid_x(c->nx, k.xout) * grid_y(c->sep.y_rows, k.by);
+    c->sep.zchunk = choose(k, tiles);
+    c->sep.grid = dim3(grid_x(c->nx, k.xout), grid_y(c->sep.y_rows, k.by), (c->nz + c->sep.zchunk - 1) / c->sep.zchunk);
+    return LBF_OK;
+  };
+  const KernelInfo none = {nullptr, 0, 0, 0, 0};
+  st = take(rows_tma ? kernel(true) : none, kernel(false), [&](const KernelInfo& k, long long tiles) {
+    const int zmax = sep_max_z(k.out_rows, c->storage);
+    if (const char* e = std::getenv("LBF_ZCHUNK")) {
+      const int v = std::atoi(e);
+      if (v >= 1) return std::min({c->nz, zmax, std::max(sep_min_z(c->nz, tiles, zmax), v)});
+    }
+    return choose_zchunk_sep(c->nz, tiles, double(sms) * resident, split ? 2.0 : 1.0, zmax);
+  });
+  if (st != LBF_OK) return st;
   // its tiles are lower than those of the 30-column kernel (FP64 2 rows against 4): lattices of more rows than
   // its grid holds keep that one
   if (!grid_fits(c->sep.grid) || (split && !grid_fits(c->grid_dirty))) return LBF_OK;
+  c->sep.ring = false;
+  if (!forced) {
+    const PlaneTime rp = ring_plane(c->Q, c->storage, c->has_mask, field, two);
+    const KernelInfo& r = c->fwd_tma30;  // the 30-column kernel, also where the line-aligned one would run
+    int rres = 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&rres, r.fn, r.threads, r.smem) != cudaSuccess)
+      return fail(LBF_ECUDA, std::string("device query failed: ") + cudaGetErrorString(cudaGetLastError()));
+    rres = std::max(rres, 1);
+    const long long rtiles = (long long)grid_x(c->nx, r.xout) * grid_y(c->ny, r.by);
+    const int rz = choose_zchunk(c->nz, rtiles, double(sms) * rres);
+    const double ring30 = estimate_us(rtiles * ((c->nz + rz - 1) / rz), sms, rres, rz + 2.0, rp);
+    double here = estimate_us((long long)c->sep.grid.x * c->sep.grid.y * c->sep.grid.z, sms, resident, c->sep.zchunk + 3.0,
+                              sep_plane(c->Q, c->storage, walls, split, field, two, small, rows_tma, c->nx));
+    if (split)  // the rows near walls run beside
+      here += (c->zchunk_dirty + 2.0) * rp.busy * double(c->grid_dirty.x) * c->grid_dirty.y * c->grid_dirty.z / sms;
+    // the line-aligned kernel, where it would run: D3Q19 0.80 to 0.89 of the 30-column kernel's time, D3Q27 0.98; the
+    // split with it 0.85 of the single masked launch
+    const double ring = ring30 * (c->aligned ? (c->Q == LBF_D3Q19 ? 0.85 : 0.98) : (split && split_by_aligned(c, p) ? 0.85 : 1.0));
+    if (1.05 * here > ring) {
+      // walls in a band of rows and a force field: the split with the 30-column kernel on both sides, FP32 only (there
+      // the masked form of that kernel is 6-8% slower, in FP64 level)
+      if (!split || !field || c->storage != LBF_F32) return LBF_OK;
+      c->sep.ring = true;
+      st = take(c->tma ? forward_for(c->Q, c->storage, false, 0, true, true, nearest) : none,
+                forward_for(c->Q, c->storage, false, 0, true, false, nearest),
+                [&](const KernelInfo&, long long tiles) { return choose_zchunk(c->nz, tiles, double(sms) * resident); });
+      if (st != LBF_OK) return st;
+      if (!grid_fits(c->sep.grid)) return LBF_OK;
+    }
+  }
+  const KernelInfo& k = c->sep.tma.fn ? c->sep.tma : c->sep.async;
   const long long blocks = (long long)c->sep.grid.x * c->sep.grid.y * c->sep.grid.z +
                            (split ? (long long)c->grid_dirty.x * c->grid_dirty.y * c->grid_dirty.z : 0);
   if (blocks > L.npartials) return fail(LBF_EINTERNAL, "partials buffer too small");
   for (int i = 0; i < 2 && c->sep.tma.fn != nullptr; ++i)
-    if ((st = encode_row_map(c, c->state[i], &c->sep.row[i], k.box_x, 1)) != LBF_OK ||
-        (st = encode_row_map(c, c->state[i], &c->sep.tile[i], k.box_x, k.by + 2)) != LBF_OK ||
-        (st = encode_row_map(c, c->state[i], &c->sep.out[i], k.box_x, k.out_rows)) != LBF_OK)
+    if ((st = sep_source_maps(c, c->state[i], &c->sep.row[i], &c->sep.tile[i])) != LBF_OK ||
+        (st = sep_store_map(c, c->state[i], &c->sep.out[i])) != LBF_OK)
       return st;
   if (split && (st = create_side(c)) != LBF_OK) return st;
   c->sep_split = split;
@@ -918,9 +1030,9 @@ lbf_status launch_sep(lbf_ctx* c, const FwdParams& a, const void* src, void* dst
   if (c->sep.tma.fn != nullptr && us % 16 == 0 && ud % 16 == 0) {  // TMA boxes start on 16-byte boundaries
     k = &c->sep.tma;
     if (ks >= 0) tr = c->sep.row[ks], tt = c->sep.tile[ks];
-    else if ((st = encode_row_map(c, src, &tr, k->box_x, 1)) == LBF_OK) st = encode_row_map(c, src, &tt, k->box_x, k->by + 2);
+    else st = sep_source_maps(c, src, &tr, &tt);
     if (st == LBF_OK && kd >= 0) to = c->sep.out[kd];
-    else if (st == LBF_OK) st = encode_row_map(c, dst, &to, k->box_x, k->out_rows);
+    else if (st == LBF_OK) st = sep_store_map(c, dst, &to);
     if (st != LBF_OK) return st;
   } else if (us % (storage_bytes(c->storage) == 8 ? 8 : 4) != 0) {  // cp.async copies 4 or 8 bytes
     return LBF_OK;
@@ -1256,7 +1368,8 @@ lbf_status lbf_create(lbf_ctx** out, const lbf_params* params, void* workspace, 
   // phase-field kernels: short chunks fill the chip on small lattices and cost the large ones nothing (the
   // restaged planes hit L2). us a step at 6 / 11 / 15 planes: droplet 128^3 113.0 / 113.7 / 114.5, layered
   // 512 x 1024 x 8 282.9 / 284.2 / 285.2, 96 x 90 x 70 59.0 / 63.7 / 68.7
-  c->zchunk_phase = std::max(std::min(6, c->nz), grid_min_z(c->nz));
+  // (FP64 is bound by its pipe: the forward step's chunks, which restage less; 70 x 60 x 50 304 us against 334)
+  c->zchunk_phase = std::max(c->storage == LBF_F64 ? c->zchunk : std::min(6, c->nz), grid_min_z(c->nz));
   c->fgrid = dim3(grid_x(c->nx, c->fwd.xout), grid_y(c->ny, c->fwd.by), (c->nz + c->zchunk - 1) / c->zchunk);
   // the adjoint marches in chunks of its own: as short as whole waves of its CTAs allow on small lattices
   // (128 x 64 x 64, us a launch at 4 / 5 / 6 / 7 / 8 planes: 34.5 / 35.7 / 26.2 / 29.7 / 32.4; 6 planes are
