@@ -640,12 +640,12 @@ int choose_zchunk_sep(int nz, long long tiles, double resident, double min_waves
 // ---- which of two kernels a step takes: the one with the shorter estimate -------------------------------------
 // A CTA takes `lone` us a plane where it has its SM to itself (latency) and adds `busy` us to an SM that runs others
 // beside it (issue, FP64 pipe, shared memory), so k resident CTAs take max(lone, k busy) us a plane together; a launch
-// runs in rounds of `resident` CTAs per SM, and many rounds run into one another. Fitted to both kernels' times on
-// 1871 lattices (2^9 to 2^27 sites, every form below) on one GB300: the estimates are within 5 to 10% of the times, the
-// choice by them is 1.3% slower than always the faster kernel. Without it, the axis-separated kernel always, 769 of
-// them were slower than with the 30-column one: tiles of 64 (FP64 32) columns waste lanes on rows of other lengths,
-// force fields (D3Q19 FP32 256^3: 424 us against 340) and FP64 walls (12 x 64 x 64: 124 against 76) cost it more, and
-// D3Q27h in FP64 is arithmetic (256^3: 27.1 ms against 23.2).
+// runs in rounds of `resident` CTAs per SM, and many rounds run into one another. Fitted to both kernels' times on 1871
+// lattices (2^9 to 2^24 sites, every form below) on one GB300, within 5 to 15%, and looked over up to 2^27 sites. Of 2238
+// lattices 26 are more than 3% slower than with the kernels there were before the axis-separated one (50 x 72 x 139 the
+// worst, 18 -> 21 us), against 613 with that kernel always: its tiles of 64 (FP64 32) columns waste lanes on rows of
+// other lengths, force fields (D3Q19 FP32 256^3: 424 us against 340) and FP64 walls (12 x 64 x 64: 124 against 76) cost
+// it more, and D3Q27h in FP64 is arithmetic (256^3: 27.1 ms against 23.2).
 struct PlaneTime {
   double lone, busy;
 };
