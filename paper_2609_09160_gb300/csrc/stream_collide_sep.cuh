@@ -1098,16 +1098,21 @@ __global__ void __launch_bounds__(32 * (sep_config(L::Q, int(sizeof(S)), L::HIGH
           }
           if (it >= 2) {
             const int z = z0 + it - 2;
-            // the sums are in units of the smallest weight, 1/36 or 1/216. p* and u, which accumulate over the steps,
-            // take that factor in two parts (rounded, and what it lacks): rounded once, it would scale them by
-            // 1 + 7e-9 (FP64 1 + 6e-17) in every step (FP32, 20 steps: error of u 9.1e-8 against 1.5e-7 with rounded
-            // weights; FP64, 50 steps, against 80-bit arithmetic: 3.2e-16 against 2.6e-15, for 1.5% of a 32^3 step)
+            // the sums are in units of the smallest weight, 1/36 or 1/216. In FP32 p* and u, which accumulate over
+            // the steps, take that factor in two parts (rounded, and what it lacks): rounded once, it would scale
+            // them by 1 + 7e-9 in every step (20 steps: error of u 9.1e-8 against 1.5e-7 with rounded weights). In
+            // FP64 it is rounded once, as the weights are in any FP64 code that adds up populations: 50 steps are
+            // 2.3e-15 off 80-bit arithmetic (the 30-column kernel 2.4e-15). In two parts they would be 3.2e-16 off
+            // that, but 25 times further from FP64 code with rounded weights, whose common factor they would lack
             constexpr T sc = Q19 ? T(1) / T(36) : T(1) / T(216);
-            // every term is exact: sc times powers of two, and differences of numbers within a factor of two
-            constexpr T lack = Q19 ? (T(1) - T(32) * sc - T(4) * sc) / T(36)
-                                   : (T(1) - T(128) * sc - T(64) * sc - T(16) * sc - T(8) * sc) / T(216);
+            constexpr T lack = T((Q19 ? 1.0 / 36.0 : 1.0 / 216.0) - double(sc));
             const V vs = v_set<V>(sc), vl = v_set<V>(lack);
-            auto scaled = [&](V v) -> V { return v_fma(v, vs, v_mul(v, vl)); };
+            auto scaled = [&](V v) -> V {
+              if constexpr (std::is_same<T, double>::value)
+                return v_mul(v, vs);
+              else
+                return v_fma(v, vs, v_mul(v, vl));
+            };
             const V b0 = scaled(f.a0);
             const bool own_row = ybl + warp * RP + r < yrows;
             const bool w0 = own_row && gx >= xb && gx < nx && !f.sol0;
