@@ -141,13 +141,11 @@ std::string kernel_name() {
 bool sep_forced(const std::string& kname) { return kname == "sep" || kname == "sepsmall"; }
 // sites below which the axis-separated kernel takes its short tile, and walls of any shape
 constexpr long long kSepSmall = 1LL << 20;
-// its masked form, the only user of the wall links and tile flags: walls with two components, on small lattices, or
-// by name. (Larger lattices are split into clean rows and rows near walls, or take the 30-column kernel)
+// its masked form, the only user of the wall links and tile flags: walls on small lattices, or by name. (Larger lattices are split into clean rows and rows near walls, or take the 30-column kernel)
 bool sep_masked(const lbf_params* p, const std::string& kname) {
   if (p->mask == nullptr || !sep_built(p)) return false;
   if (sep_forced(kname)) return true;
-  const bool small = (long long)p->nx * p->ny * p->nz < kSepSmall && storage_bytes(p->storage) != 2;
-  return kname.empty() && (p->two_component || small);
+  return kname.empty() && !p->two_component && (long long)p->nx * p->ny * p->nz < kSepSmall && storage_bytes(p->storage) != 2;
 }
 // z-chunks of the axis-separated kernel: at most kSepMaxZ planes (64 with one FP32 row per warp, whose threads add
 // up their sums over a whole chunk), at least two and no fewer than keep a grid of `tiles` columns within
@@ -655,14 +653,12 @@ double estimate_us(long long blocks, int sms, int resident, double planes, Plane
   if (full >= 4) return planes * round * (double(blocks) / (double(sms) * resident) + 0.3);
   return planes * (full * round + (rest > 0 ? std::max(p.lone, p.busy * rest) : 0.0));
 }
-// the 30-column kernel (two: 1 equal densities, 2 a density contrast)
-PlaneTime ring_plane(int lattice, int storage, bool walls, bool field, int two) {
+// the 30-column kernel
+PlaneTime ring_plane(int lattice, int storage, bool walls, bool field) {
   if (storage == LBF_F64) {  // the FP64 pipe
     const double t = (lattice == LBF_D3Q19 ? 7.2 : (lattice == LBF_D3Q27 ? 9.5 : 21.5)) * (field ? 1.04 : 1.0);
     return {t, t};
   }
-  if (two == 1) return walls ? PlaneTime{2.26, 1.13} : PlaneTime{1.63, 0.84};
-  if (two == 2) return walls ? PlaneTime{2.87, 1.40} : PlaneTime{1.93, 1.02};
   PlaneTime p = {1.12, 0.76};  // D3Q27h
   if (lattice == LBF_D3Q19) p = walls ? PlaneTime{1.0, 0.70} : PlaneTime{0.87, 0.60};
   if (lattice == LBF_D3Q27) p = walls ? PlaneTime{1.22, 0.87} : PlaneTime{0.87, 0.54};
@@ -670,16 +666,13 @@ PlaneTime ring_plane(int lattice, int storage, bool walls, bool field, int two) 
   return p;
 }
 // the axis-separated kernel: walls in its masked form, or the clean rows of a split step
-PlaneTime sep_plane(int lattice, int storage, bool walls, bool split, bool field, int two, bool small, bool rows_tma, int nx) {
+PlaneTime sep_plane(int lattice, int storage, bool walls, bool split, bool field, bool small, bool rows_tma, int nx) {
   PlaneTime p;
   double f = 1.0;
   if (storage == LBF_F64) {
     const double t = lattice == LBF_D3Q19 ? (walls ? 5.1 : 3.7) : (lattice == LBF_D3Q27 ? (walls ? 6.7 : 5.0) : 14.0);
     p = {t, t};
     f = (field && !walls ? 1.13 : 1.0) * (rows_tma ? 1.0 : 1.08);
-  } else if (two != 0) {
-    p = two == 1 ? (walls ? PlaneTime{2.9, 1.65} : PlaneTime{2.44, 1.35}) : (walls ? PlaneTime{3.4, 2.1} : PlaneTime{2.7, 1.65});
-    f = rows_tma ? 1.0 : 1.25;
   } else if (small) {
     p = {1.14, 1.08};  // D3Q27h
     if (lattice == LBF_D3Q19) p = walls ? PlaneTime{0.70, 0.62} : PlaneTime{0.45, 0.41};
@@ -875,6 +868,10 @@ lbf_status setup_sep(lbf_ctx* c, const lbf_params* p, const Layout& L, int sms, 
   // grow only with what drives the flow (that cancel where nothing does). No lattice size brings that below FP32
   // rounding for every n, so the axis-separated kernel is taken here only on request (LBF_KERNEL=sep, sepsmall)
   if (storage_bytes(c->storage) == 2 && !forced) return LBF_OK;
+  // two components keep the 30-column kernel as well: where grad phi is small its direction, which drives the interface
+  // flux, hangs on the last bits of u, and 50 steps of a 128^3 droplet end up to 6e-5 of phi apart (its error against
+  // FP64: 5e-5). This kernel is 1.10 times faster there and on request only
+  if (c->two && !forced) return LBF_OK;
   const bool field = p->force_field != nullptr;
   // below about 2^20 sites the tall tiles leave SMs idle: short ones (ensemble members, 524288 sites with
   // walls and a force field: 17 us a step against 20.6)
@@ -882,7 +879,7 @@ lbf_status setup_sep(lbf_ctx* c, const lbf_params* p, const Layout& L, int sms, 
   const bool rows_tma = tma_eligible(c->storage, c->nx) && c->nx >= 32 * sep_vx(int(storage_bytes(c->storage)));
   // large lattices whose rows TMA cannot take: the 30-column kernel (333 x 250 x 189, GLUPS: 38.0 against
   // 34.8 with the best tile of this one)
-  if (!rows_tma && !small && !forced && !c->two) return LBF_OK;
+  if (!rows_tma && !small && !forced) return LBF_OK;
   bool walls = c->has_mask, split = false;
   c->sep.y_begin = 0;
   c->sep.y_rows = c->ny;
@@ -891,7 +888,7 @@ lbf_status setup_sep(lbf_ctx* c, const lbf_params* p, const Layout& L, int sms, 
     return two ? sep_two_kernel_for(c->Q, c->storage, walls, two, tma)
                : sep_kernel_for(c->Q, c->storage, walls, field, tma, nearest, small);
   };
-  if (walls && kname.empty() && !small && !two) {
+  if (walls && kname.empty() && !small) {
     const KernelInfo k = sep_kernel_for(c->Q, c->storage, false, field, false, nearest, small);
     int begin = 0, len = 0;
     if (!clean_band(c, p, k.by, &begin, &len)) return LBF_OK;  // scattered walls: the 30-column
@@ -937,7 +934,7 @@ lbf_status setup_sep(lbf_ctx* c, const lbf_params* p, const Layout& L, int sms, 
   if (!grid_fits(c->sep.grid) || (split && !grid_fits(c->grid_dirty))) return LBF_OK;
   c->sep.ring = false;
   if (!forced) {
-    const PlaneTime rp = ring_plane(c->Q, c->storage, c->has_mask, field, two);
+    const PlaneTime rp = ring_plane(c->Q, c->storage, c->has_mask, field);
     const KernelInfo& r = c->fwd_tma30;  // the 30-column kernel, also where the line-aligned one would run
     int rres = 1;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&rres, r.fn, r.threads, r.smem) != cudaSuccess)
@@ -947,7 +944,7 @@ lbf_status setup_sep(lbf_ctx* c, const lbf_params* p, const Layout& L, int sms, 
     const int rz = choose_zchunk(c->nz, rtiles, double(sms) * rres);
     const double ring30 = estimate_us(rtiles * ((c->nz + rz - 1) / rz), sms, rres, rz + 2.0, rp);
     double here = estimate_us((long long)c->sep.grid.x * c->sep.grid.y * c->sep.grid.z, sms, resident, c->sep.zchunk + 3.0,
-                              sep_plane(c->Q, c->storage, walls, split, field, two, small, rows_tma, c->nx));
+                              sep_plane(c->Q, c->storage, walls, split, field, small, rows_tma, c->nx));
     if (split)  // the rows near walls run beside
       here += (c->zchunk_dirty + 2.0) * rp.busy * double(c->grid_dirty.x) * c->grid_dirty.y * c->grid_dirty.z / sms;
     // the line-aligned kernel, where it would run: D3Q19 0.80 to 0.89 of the 30-column kernel's time, D3Q27 0.98; the

@@ -183,6 +183,8 @@ __global__ void k_reduce_final(const double* __restrict__ partials, long long nb
 // z-filtered values, and the outputs apply the x-y filters from it. What bounds them is latency (128^3: one
 // wave of CTAs, 6 per SM, marching 17 planes): the plane's shared memory is double, so a plane has one
 // barrier.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 struct PhaseParams {
   int nx, ny, nz;
   long long N;
@@ -244,6 +246,9 @@ struct PhaseColumn {
 // phi_new from phi, u (decoded from the state) and G, all at time n:
 //   phi' = phi - 3 sum_i w_i c_i . V(x + c_i) + 6 D sum_i w_i (phi(x + c_i) - phi(x)),
 //   V = phi u + lambda G
+// The flux and its average along z are written with their roundings (fma, mul_rn): left to the compiler, the planes
+// before a chunk's first and those of its loop were contracted differently, so phi depended on where chunks begin; by
+// the last bit, but the direction grad phi / |grad phi| turns that into up to 6e-5 of phi in 50 steps of a droplet.
 // With walls, u is taken as 0 at solid sites and phi is not advanced there (it keeps its value),
 // so a wall in contact with one bulk phase exchanges no phi.
 template <class S, class T>
@@ -280,9 +285,9 @@ __global__ void __launch_bounds__(PhaseTile<T>::SITES, sizeof(T) == 4 ? 6 : 1)
   };
   auto take = [&](int k, const Raw& r) {
     f[k] = r.ph;
-    vx[k] = r.ph * r.ux + lam * r.gx;
-    vy[k] = r.ph * r.uy + lam * r.gy;
-    vz[k] = r.ph * r.uz + lam * r.gz;
+    vx[k] = fma(lam, r.gx, mul_rn(r.ph, r.ux));
+    vy[k] = fma(lam, r.gy, mul_rn(r.ph, r.uy));
+    vz[k] = fma(lam, r.gz, mul_rn(r.ph, r.uz));
   };
   Raw r0, r1;
   fetch(c.z0 - 1, r0);
@@ -296,8 +301,8 @@ __global__ void __launch_bounds__(PhaseTile<T>::SITES, sizeof(T) == 4 ? 6 : 1)
     T(*const b)[PT::SITES] = sm[(z - c.z0) & 1];
     b[0][me] = f[1];
     b[1][me] = PT::A1 * ((f[0] - f[1]) + (f[2] - f[1]));
-    b[2][me] = PT::A0 * vx[1] + PT::A1 * (vx[0] + vx[2]);
-    b[3][me] = PT::A0 * vy[1] + PT::A1 * (vy[0] + vy[2]);
+    b[2][me] = fma(PT::A0, vx[1], mul_rn(PT::A1, vx[0] + vx[2]));
+    b[3][me] = fma(PT::A0, vy[1], mul_rn(PT::A1, vy[0] + vy[2]));
     b[4][me] = PT::A1 * (vz[2] - vz[0]);
     __syncthreads();
     if (c.out) {
