@@ -553,15 +553,16 @@ def kernel_label(s, lattice, storage, kind):
     """The kernels one timed step runs (the roofline unit is one step: its launches together)."""
     lat = LATTICE_NAME[lattice]
     walls = kind in ("channel", "layered")
+    wide = storage in ("f32", "f64")
     if s.kernels_per_step == 2 and kind == "channel":
-        return (f"k_stream_collide_sep<{lat},{storage},periodic> on the rows clear of the walls + "
+        clean = "k_stream_collide_sep" if wide else "k_stream_collide_al"
+        return (f"{clean}<{lat},{storage},periodic> on the rows clear of the walls + "
                 f"k_stream_collide<{lat},{storage},mask> on the rows near them")
-    if storage in ("f16", "bf16") and kind == "tg256":
-        return f"k_stream_collide or k_stream_collide_al<{lat},{storage},periodic> (the library's choice)"
-    fused = f"k_stream_collide_sep<{lat},{storage},{'mask' if walls else 'periodic'}>"
     if kind in ("droplet", "layered"):
-        return f"k_phase_advance + k_phase_forces + {fused}"
-    return fused
+        return f"k_phase_advance + k_phase_forces + k_stream_collide<{lat},{storage},{'mask' if walls else 'periodic'}>"
+    if not wide:
+        return f"k_stream_collide or k_stream_collide_al<{lat},{storage},{'mask' if walls else 'periodic'}> (the library's choice)"
+    return f"k_stream_collide_sep<{lat},{storage},{'mask' if walls else 'periodic'}>"
 
 
 def run_ours(args):

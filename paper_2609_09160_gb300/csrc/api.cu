@@ -360,8 +360,8 @@ const void* mapped_host_pointer(const void* p) {
 // A launch whose start may overlap the end of the kernel before it in the stream (programmatic dependent
 // launch); the kernel calls grid_wait() before it touches memory. It hides the launch and start-up of the
 // step's kernels (us a step, before -> after: 64 x 48 x 40 channel 10.3 -> 7.3, 524288 sites with a force
-// field 18.0 -> 15.7, droplet 128^3 113 -> 107). From about 2^23 sites on, grids of many waves gain nothing
-// and their first wave settles less evenly (512^3 FP16 1409 -> 1426), so those are launched as usual.
+// field 18.0 -> 15.7): some 2 us, which is 4 to 10% at 2^20 sites, 1 to 2% at 2^23, under 0.5% from 2^25 on (both step
+// kernels, walls, 16-bit, two components). Launches of 2^23 sites and more are left as usual.
 cudaError_t launch_overlapped(const void* fn, dim3 grid, dim3 block, void** args, size_t smem, cudaStream_t st,
                               long long sites) {
   if (sites >= (1LL << 23)) return cudaLaunchKernel(fn, grid, block, args, smem, st);
@@ -640,7 +640,7 @@ int choose_zchunk_sep(int nz, long long tiles, double resident, double min_waves
 // beside it (issue, FP64 pipe, shared memory), so k resident CTAs take max(lone, k busy) us a plane together; a launch
 // runs in rounds of `resident` CTAs per SM, and many rounds run into one another. Fitted to both kernels' times on 1871
 // lattices (2^9 to 2^24 sites, every form below) on one GB300, within 5 to 15%, and looked over up to 2^27 sites. Of 2238
-// lattices 26 are more than 3% slower than with the kernels there were before the axis-separated one (50 x 72 x 139 the
+// lattices 18 are more than 3% slower than with the kernels there were before the axis-separated one (50 x 72 x 139 the
 // worst, 18 -> 21 us), against 613 with that kernel always: its tiles of 64 (FP64 32) columns waste lanes on rows of
 // other lengths, force fields (D3Q19 FP32 256^3: 424 us against 340) and FP64 walls (12 x 64 x 64: 124 against 76) cost
 // it more, and D3Q27h in FP64 is arithmetic (256^3: 27.1 ms against 23.2).
@@ -1362,11 +1362,13 @@ lbf_status lbf_create(lbf_ctx** out, const lbf_params* params, void* workspace, 
     if (v >= 1) zc = std::max(min_zchunk(c->nz), v);
   }
   c->zchunk = std::min(zc, c->nz);
-  // phase-field kernels: short chunks fill the chip on small lattices and cost the large ones nothing (the
-  // restaged planes hit L2). us a step at 6 / 11 / 15 planes: droplet 128^3 113.0 / 113.7 / 114.5, layered
-  // 512 x 1024 x 8 282.9 / 284.2 / 285.2, 96 x 90 x 70 59.0 / 63.7 / 68.7
-  // (FP64 is bound by its pipe: the forward step's chunks, which restage less; 70 x 60 x 50 304 us against 334)
-  c->zchunk_phase = std::max(c->storage == LBF_F64 ? c->zchunk : std::min(6, c->nz), grid_min_z(c->nz));
+  // phase-field kernels, whose values do not depend on the chunks: short ones fill the chip on small lattices (us a step
+  // at 6 / 11 / 15 planes: 96 x 90 x 70 59.0 / 63.7 / 68.7) and suit a density contrast on large ones, where grad phi is
+  // written as well (400^3 at 6 / 12 / 24: 3891 / 3904 / 3960); equal densities from about 2^21 sites on take 12 planes,
+  // which restage less (at 6 / 12 / 24: 128^3 117.6 / 115.7 / 125.0, 256^3 843 / 824 / 824). FP64 is bound by its pipe:
+  // the forward step's chunks (70 x 60 x 50 304 us against 334 at 6)
+  c->zchunk_phase = c->storage == LBF_F64 ? c->zchunk : std::min(c->nz, !c->contrast && c->N >= (1LL << 21) ? 12 : 6);
+  c->zchunk_phase = std::max(c->zchunk_phase, grid_min_z(c->nz));
   c->fgrid = dim3(grid_x(c->nx, c->fwd.xout), grid_y(c->ny, c->fwd.by), (c->nz + c->zchunk - 1) / c->zchunk);
   // the adjoint marches in chunks of its own: as short as whole waves of its CTAs allow on small lattices
   // (128 x 64 x 64, us a launch at 4 / 5 / 6 / 7 / 8 planes: 34.5 / 35.7 / 26.2 / 29.7 / 32.4; 6 planes are

@@ -601,8 +601,7 @@ __global__ void __launch_bounds__(FwdTile<BY>::THREADS, fwd_minb(L::Q, int(sizeo
   constexpr int G0 = D::gsize(0) * SITES, G1 = D::gsize(1) * SITES, G2 = D::gsize(2) * SITES;
   constexpr int GS2 = D::gsize(2);  // three-slot offsets: ring g2 = slot * G2, solid flags g2 / GS2
   constexpr bool SITEF = TWO || FF;  // per-site force (else the uniform force of the parameters)
-  static_assert(fwd_smem_bytes<L, S, BY, MASK, TMA>() >= 6 * 512 * sizeof(double), "smem too small for the final tree");
-  static_assert(FwdTile<BY>::THREADS <= 512, "final tree assumes <= 512 threads");
+  static_assert(fwd_smem_bytes<L, S, BY, MASK, TMA>() >= 6 * (FwdTile<BY>::THREADS / 32) * sizeof(double), "smem too small for sum_partials");
 
   extern __shared__ __align__(128) unsigned char smem_raw[];
   S* rawst = reinterpret_cast<S*>(smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u));

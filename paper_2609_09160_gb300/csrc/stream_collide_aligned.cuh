@@ -151,8 +151,7 @@ __global__ void __launch_bounds__(AlTile<S, TY>::THREADS, al_minb<L, S, TY, MASK
   constexpr int GS2 = D::gsize(2);
   constexpr int OSTR = TY * 32;  // field stride of the output stage
   constexpr int OSTAGE = int(round128(size_t(10) * TY * 32 * sizeof(S)) / sizeof(S));  // elements per output stage
-  static_assert(al_smem_bytes<L, S, TY, MASK>() >= 6 * 512 * sizeof(double) + 128, "smem too small for the final tree");
-  static_assert(G::THREADS <= 512, "final tree assumes <= 512 threads");
+  static_assert(al_smem_bytes<L, S, TY, MASK>() >= 6 * (G::THREADS / 32) * sizeof(double) + 128, "smem too small for sum_partials");
 
   extern __shared__ __align__(128) unsigned char smem_raw[];
   unsigned char* sbase = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);

@@ -33,10 +33,11 @@
 // is moved left to end at nx - 1. Rows that are not whole 16-byte units, or shorter than a tile, are
 // loaded into registers one plane ahead as well.
 //
-// What bounds it (one GB300; GLUPS, same workloads, before -> after; "before" is the faster of the two
-// population-ring kernels):
-//   D3Q19 FP32 512^3 64.6 -> 70, 256^3 57.0 -> 67; FP16 512^3 65.5 -> 94; D3Q27 FP32 512^3 51.8 -> 64,
-//   FP16 53.6 -> 71.5; D3Q27h FP32 256^3 31.6 -> 39.4, FP16 29.8 -> 38.7; D3Q19 FP64 32^3 0.43 -> 1.13.
+// What bounds it (one GB300; us a step, steps without sums; "before" is the faster of the two population-ring kernels):
+//   D3Q19 FP32 512^3 2024 -> 1895, 256^3 280 -> 248, 128^3 52 -> 37, 32^3 12.4 -> 4.5; D3Q27 FP32 512^3 2523 -> 2071,
+//   256^3 354 -> 270; D3Q27h FP32 512^3 3923 -> 3283, 256^3 535 -> 425; D3Q19 FP64 32^3 75.9 -> 29.5, 256^3 7668 -> 6968.
+//   By name only (16-bit storage and two components keep the ring kernels' values): D3Q19 FP16 512^3 with its sums 2043 ->
+//   1448, D3Q27 FP16 2500 -> 1973, droplet 128^3 116 -> 107.
 //   Thread instructions per site: D3Q19 FP32 188 (421 before), FP16 245, D3Q27 FP32 305 (600), D3Q27h 460
 //   (970). FP32 moves DRAM at 5.6 TB/s of 6.7 (reads 1.03x the state); 16-bit storage and the D3Q27 lattices
 //   are bound by the latency of the two halves of a plane's work with 8 to 16 warps per SM (shared-memory
@@ -49,7 +50,7 @@
 //     CTA per SM with 5 stages of 8 rows (72) over two of 6 rows with 4 (67).
 //   * outputs leave as TMA boxes from the stage rows just read: 62.6 -> 68.6 (FP32 256^3) against per-thread
 //     stores, which queue in front of the other warps' shared-memory accesses.
-//   * two components (TWO): the forces and phase field of the source and of the output sites are loaded as
+//   * two components (TWO, by name): the forces and phase field of the source and of the output sites are loaded as
 //     pairs one plane ahead: droplet 128^3 72 -> 56 us a launch against scalar loads (83 before), layered
 //     contrast flow 205 -> 175; 8 warps of 126 registers, two CTAs per SM (6 warps 118, here 115 us a step).
 //   * rows 0 and TY + 1 and the halo columns on two warps of their own: the warp that carried both took
