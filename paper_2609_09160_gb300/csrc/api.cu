@@ -640,7 +640,7 @@ int choose_zchunk_sep(int nz, long long tiles, double resident, double min_waves
 // beside it (issue, FP64 pipe, shared memory), so k resident CTAs take max(lone, k busy) us a plane together; a launch
 // runs in rounds of `resident` CTAs per SM, and many rounds run into one another. Fitted to both kernels' times on 1871
 // lattices (2^9 to 2^24 sites, every form below) on one GB300, within 5 to 15%, and looked over up to 2^27 sites. Of 2238
-// lattices 18 are more than 3% slower than with the kernels there were before the axis-separated one (50 x 72 x 139 the
+// lattices 12 are more than 3% slower than with the kernels there were before the axis-separated one (50 x 72 x 139 the
 // worst, 18 -> 21 us), against 613 with that kernel always: its tiles of 64 (FP64 32) columns waste lanes on rows of
 // other lengths, force fields (D3Q19 FP32 256^3: 424 us against 340) and FP64 walls (12 x 64 x 64: 124 against 76) cost
 // it more, and D3Q27h in FP64 is arithmetic (256^3: 27.1 ms against 23.2).
@@ -943,10 +943,12 @@ lbf_status setup_sep(lbf_ctx* c, const lbf_params* p, const Layout& L, int sms, 
     const long long rtiles = (long long)grid_x(c->nx, r.xout) * grid_y(c->ny, r.by);
     const int rz = choose_zchunk(c->nz, rtiles, double(sms) * rres);
     const double ring30 = estimate_us(rtiles * ((c->nz + rz - 1) / rz), sms, rres, rz + 2.0, rp);
-    double here = estimate_us((long long)c->sep.grid.x * c->sep.grid.y * c->sep.grid.z, sms, resident, c->sep.zchunk + 3.0,
-                              sep_plane(c->Q, c->storage, walls, split, field, small, rows_tma, c->nx));
-    if (split)  // the rows near walls run beside
-      here += (c->zchunk_dirty + 2.0) * rp.busy * double(c->grid_dirty.x) * c->grid_dirty.y * c->grid_dirty.z / sms;
+    auto grid_us = [&](double planes, PlaneTime t) {
+      return estimate_us((long long)c->sep.grid.x * c->sep.grid.y * c->sep.grid.z, sms, resident, planes, t);
+    };
+    // the rows near walls of a split run beside
+    const double beside = !split ? 0.0 : (c->zchunk_dirty + 2.0) * rp.busy * double(c->grid_dirty.x) * c->grid_dirty.y * c->grid_dirty.z / sms;
+    const double here = beside + grid_us(c->sep.zchunk + 3.0, sep_plane(c->Q, c->storage, walls, split, field, small, rows_tma, c->nx));
     // the line-aligned kernel, where it would run: D3Q19 0.80 to 0.89 of the 30-column kernel's time, D3Q27 0.98; the
     // split with it 0.85 of the single masked launch
     const double ring = ring30 * (c->aligned ? (c->Q == LBF_D3Q19 ? 0.85 : 0.98) : (split && split_by_aligned(c, p) ? 0.85 : 1.0));
@@ -959,7 +961,9 @@ lbf_status setup_sep(lbf_ctx* c, const lbf_params* p, const Layout& L, int sms, 
                 forward_for(c->Q, c->storage, false, 0, true, false, nearest),
                 [&](const KernelInfo&, long long tiles) { return choose_zchunk(c->nz, tiles, double(sms) * resident); });
       if (st != LBF_OK) return st;
-      if (!grid_fits(c->sep.grid)) return LBF_OK;
+      // the second launch and the join cost some 3 us, and the estimates of the two forms are near each other
+      const double both = 3.0 + beside + grid_us(c->sep.zchunk + 2.0, ring_plane(c->Q, c->storage, false, field));
+      if (!grid_fits(c->sep.grid) || 1.1 * both > ring30) return LBF_OK;
     }
   }
   const KernelInfo& k = c->sep.tma.fn ? c->sep.tma : c->sep.async;

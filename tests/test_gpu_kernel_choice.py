@@ -76,7 +76,7 @@ def test_default_step_is_not_slower_than_the_30_column_kernel(case):
 
 @pytest.mark.parametrize("lattice", [19, 27])
 def test_split_with_a_force_field_matches_the_single_launch(lattice):
-    for shape in ((34, 130, 260), (17, 260, 260), (33, 131, 261)):
+    for shape in ((34, 130, 260), (68, 130, 260), (33, 131, 261)):
         c = dict(lattice=lattice, storage="f32", shape=shape, field=True, walls="band")
         a, b = _solver(None, c), _solver("cta", c)
         assert a.kernels_per_step == 2 or shape[2] % 2
